@@ -3,21 +3,21 @@
 // A persistent grid takes targets (cells) from a job list: a job is one
 // built tree and a range or list of its cells, so one launch can serve
 // several independent problems.
-// Walk (Sec. 2.3-2.4): the CTA keeps a stack of opened nodes in shared
-// memory.  Each step pops up to NT/8 opened nodes and evaluates their NT
+// Walk (Sec. 2.3-2.4): the CTA keeps the opened nodes in a ring buffer in
+// shared memory.  Each step takes up to NT/8 of them and evaluates their NT
 // children at once, one child per thread: a child that contains the target,
 // or fails the BH MAC (h/d < theta_lim), the IF MAC (nodes holding an
 // ionisation front: h/d < theta_IF) or the Src MAC (emitting nodes:
-// h/d < theta_src), is pushed as opened; the others are accepted.  On an
-// AMR tree a node flagged as a cell is never opened.
+// h/d < theta_src), is pushed as opened; the others are accepted and listed.
+// On an AMR tree a node flagged as a cell is never opened.
 // In the FP32 forms the distances come from FP32 records, and every opening
 // decision and every discontinuous choice of the radial spreading (beyond
 // L_ray or not, beyond the last point or not, a kernel support that is empty
 // or holds one point) that FP32 cannot settle within a certified bound on
 // its distance error is re-taken in FP64 from an FP64 copy of the tree: the
 // accepted nodes are those of the FP64 form, bit for bit.
-// Map (Sec. 2.3, App. A): the nodes accepted in a step are spread by the
-// whole CTA over the rays their table entry lists (angular weights) and the
+// Map (Sec. 2.3, App. A): the warps spread the listed nodes, 32 at a time,
+// over the rays their table entry lists (angular weights) and the
 // evaluation points their radial kernel reaches (W_p or W_g for the
 // recombination rate alpha and the energy e; W_f,3 or another flux kernel
 // for the emission eps), with shared-memory atomics into the ray bins: FP64
@@ -26,10 +26,10 @@
 // FP32 + FP64-sweep forms: a thread per ray, FP64 arithmetic; FP32 +
 // double-FP32-sweep form: two lanes per ray, FP32 losses, double-FP32
 // budgets) and the CTA sums the rays (Eq. 18).
-// Variants: wide CTAs (512 / 256 threads) when the bins fill an SM, a
-// register-capped walk when six CTAs fit, a dump mode keeping the raw bins
-// and accepted ids, a column-density mode without radial points, and a
-// separate instantiation for non-default kernels and boundaries.
+// Variants: CTAs of 128, 256 or 512 threads by the room that the bins leave,
+// a dump mode keeping the raw bins and accepted ids, a column-density mode
+// without radial points, and a separate instantiation for non-default
+// kernels and boundaries.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -53,7 +53,7 @@ struct WalkArgs {
     const void* nodes;
     const NodeF64* nodes64;                 // FP32 forms: the FP64 tree (exact re-decisions)
     const float* kappa;                     // FP32 forms: |cm32 - cm64| <= kappa x edge
-    int N, L, nr, npix, eta, nside, use_e, stack_cap;
+    int N, L, nr, npix, eta, nside, use_e;
     double th_lim2, th_if2, th_src2, lray;
     double r_coef;                          // r_i = i^2 r_coef cells, r_coef = 1 / (2 eta^2) (Eq. 4)
     float r_coeff;                          // the same (a power of two: exact in FP32)
@@ -161,46 +161,50 @@ __device__ __forceinline__ void bc_frame(int bc, int mirrored, int N, int g2, in
     }
 }
 
-__device__ __forceinline__ int face_bin(int x, int A) {
-    if (x == 0) return TQH;
-    int q = (TQH * abs(x)) / A;
-    q = min(q, TQH - 1);
-    return x > 0 ? TQH + 1 + q : TQH - 1 - q;
+// Bin of face coordinate x / A (|x| < A or, on a tie, the last bin): floor(16
+// |x| / A) from one approximate reciprocal rA of A.  (16 |x| + 1/2) / A lies
+// at least 1 / (2A) >= 2.4e-4 from an integer (A < 2048) and the product is
+// off by less than 1e-5, so the floor is exact without an integer division.
+__device__ __forceinline__ int face_bin(int x, float rA) {
+    const int q = min((int)(fmaf((float)abs(x), (float)TQH, 0.5f) * rA), TQH - 1);
+    return x == 0 ? TQH : (x > 0 ? TQH + 1 + q : TQH - 1 - q);
 }
 
 // Table key of a node from the integer offset o = 2 (node centre - target
 // centre) in half cells and the node edge s in cells: a face key when one
 // axis has the largest |o|, an edge key when two tie for it, a corner key
-// when all three do.
+// when all three do.  psi bin = floor(64 s / |o|), at most TB - 1: FP32 gives
+// it to 3e-5, so the exact integer comparison is made only within 1e-4 of an
+// integer (a bin in ten thousand).
 __device__ __forceinline__ int table_key(int ox, int oy, int oz, int s) {
     const int ax = abs(ox), ay = abs(oy), az = abs(oz);
     const int A = max(ax, max(ay, az));
-    const long long o2 = (long long)ox * ox + (long long)oy * oy + (long long)oz * oz;
-    const long long lim = 64LL * s, lim2 = lim * lim;
-    long long pb = (long long)((float)lim * rsqrtf((float)o2));
-    while (pb > 0 && pb * pb * o2 > lim2) --pb;
-    while ((pb + 1) * (pb + 1) * o2 <= lim2) ++pb;
-    if (pb > TB - 1) pb = TB - 1;
-    const int tx = ax == A, ty = ay == A, tz = az == A;
-    const int ntie = tx + ty + tz;
+    const int o2 = ox * ox + oy * oy + oz * oz;              // < 3 x 2048^2: exact, also as a float
+    const float q = 64.f * (float)s * rsqrtf((float)o2);
+    int pb = (int)fminf(q, (float)(TB - 1));
+    if (q < (float)TB && fabsf(q - rintf(q)) < 1e-4f) {
+        const long long lim = 64LL * s, lim2 = lim * lim;
+        if ((long long)pb * pb * o2 > lim2) --pb;
+        else if ((long long)(pb + 1) * (pb + 1) * o2 <= lim2) ++pb;
+        pb = min(pb, TB - 1);
+    }
+    const float rA = __fdividef(1.f, (float)A);
+    const bool tx = ax == A, ty = ay == A, tz = az == A;
+    const int ntie = (int)tx + (int)ty + (int)tz;
     if (ntie == 1) {
-        const int a = tx ? 0 : (ty ? 1 : 2);
-        const int ob = (a == 0) ? oy : ox;
-        const int oc = (a == 2) ? oy : oz;
-        const int oa = (a == 0) ? ox : (a == 1 ? oy : oz);
-        const int face = 2 * a + (oa < 0 ? 1 : 0);
-        const int u = face_bin(ob, A), v = face_bin(oc, A);
-        return ((face * TQ + u) * TQ + v) * TB + (int)pb;
+        const int ob = tx ? oy : ox, oc = tz ? oy : oz, oa = tx ? ox : (ty ? oy : oz);
+        const int face = (tx ? 0 : (ty ? 2 : 4)) + (oa < 0 ? 1 : 0);
+        return ((face * TQ + face_bin(ob, rA)) * TQ + face_bin(oc, rA)) * TB + pb;
     }
     if (ntie == 2) {                         // edge of the tied axes a < b, the third axis c binned
         const int c = !tx ? 0 : (!ty ? 1 : 2);
         const int pair = c == 2 ? 0 : (c == 1 ? 1 : 2);
         const int oa = c == 0 ? oy : ox, ob = c == 2 ? oy : oz, oc = c == 0 ? ox : (c == 1 ? oy : oz);
         const int edge = 4 * pair + 2 * (oa < 0) + (ob < 0);
-        return NFACEKEYS + (edge * TQ + face_bin(oc, A)) * TB + (int)pb;
+        return NFACEKEYS + (edge * TQ + face_bin(oc, rA)) * TB + pb;
     }
     const int corner = (ox < 0) + 2 * (oy < 0) + 4 * (oz < 0);
-    return NFACEKEYS + NEDGEKEYS + corner * TB + (int)pb;
+    return NFACEKEYS + NEDGEKEYS + corner * TB + pb;
 }
 
 // Ray bins.  FP64 form: one double per bin, atomic FP64 adds.  FP32 form: the
@@ -237,21 +241,29 @@ __device__ __forceinline__ bool bin_nonzero(const double* slot) {
     return (v.x | v.y) != 0u;
 }
 
+// FP32 forms: add v >= 0 (in units of the bin, below 2^62), rounded down to an
+// integer, to a bin.  Integer placement of the significand rather than two
+// float-to-integer conversions: those share a pipe of 16 lanes per SM and
+// clock (turbulent128, double-FP32 form: 232 -> 226 ms; the unconditional
+// second atomic 226 -> 217 ms).
+__device__ __forceinline__ void bin_add_units(double* slot, float v) {
+    unsigned* w = reinterpret_cast<unsigned*>(slot);
+    // the 24-bit significand placed in 64 bits by one widening multiply
+    const uint32_t b = __float_as_uint(v);
+    const int t = (int)(b >> 23) - 126;                       // v in [2^(t-1), 2^t)
+    const uint64_t p = (uint64_t)((b << 8) | 0x80000000u) * (1u << (t & 31));
+    const uint32_t pl = (uint32_t)p, ph = (uint32_t)(p >> 32);
+    const uint32_t lo = t >= 32 ? pl : (t > 0 ? ph : 0u), hi = t >= 32 ? ph : 0u;
+    const unsigned old = atomicAdd(w, lo);
+    unsigned h;
+    asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\taddc.u32 %0, %3, 0;\n\t}" : "=r"(h) : "r"(old), "r"(lo), "r"(hi));
+    atomicAdd(w + 1, h);                                      // (a branch around zero costs more)
+}
+
 template <int MODE>
 __device__ __forceinline__ void bin_atomic_add(double* slot, typename Prec<MODE>::real x, float scale) {
-    if (MODE == 0) {
-        atomicAdd(slot, (double)x);
-    } else {
-        const float v = (float)x * scale;                     // exact: scale is a power of two
-        if (!(v > 0.f)) return;
-        const float hf = floorf(v * 2.3283064365386963e-10f);  // v / 2^32, exact
-        const float lf = v - hf * 4294967296.0f;              // exact, < 2^32
-        const unsigned lo = (unsigned)lf, hi = (unsigned)hf;
-        unsigned* w = reinterpret_cast<unsigned*>(slot);
-        const unsigned old = atomicAdd(w, lo);
-        const unsigned carry = (old + lo < old) ? 1u : 0u;
-        if (hi + carry) atomicAdd(w + 1, hi + carry);
-    }
+    if constexpr (MODE == 0) atomicAdd(slot, (double)x);
+    else bin_add_units(slot, (float)x * scale);               // exact: scale is a power of two
 }
 
 template <int MODE>
@@ -333,23 +345,40 @@ __device__ __forceinline__ double exact_d2(const WalkArgs& a, int64_t nid, float
     return dist2((double)tx, (double)ty, (double)tz, cm);
 }
 
-// Radial spread of one accepted node (App. A), prepared by the thread that
-// accepted it and applied by the whole CTA, one (node, ray) pair per thread.
-// kind 0: W_p(|r_i - d| / h) / S over points lo .. lo+npts-1 (S = sum over
-// all points); kind 1: everything on one point (node beyond the last point);
-// kind 2: linear split w0, w1 between the two points bracketing d (no point
-// inside the W_p support).
+// Radial spread of one accepted node (App. A), prepared by one lane: the
+// points lo .. lo+npts-1 and their weights.  The weights are the values that
+// the lane keeps in its column of the warp's NodeBatch, times b; a support
+// of more than MAXW points is evaluated again for each ray instead (`lng`:
+// column entries 0 and 1 then hold d and the kernel's size argument).
+// Kernel values kept per node.  FP32: 8, so that five CTAs fit an SM beside
+// 33 KB of ray bins (N_PIX 48, N_R 43; with 12 only four do: 225 -> 253 ms);
+// a longer support, met by the few nodes with edges of 32 cells and more,
+// costs its evaluation again per ray.  FP64: 12, evaluating again costs more.
+template <int MODE> constexpr int MAXW = MODE == 0 ? 12 : 8;
+
 template <int MODE>
 struct RadialSpread {
-    typename Prec<MODE>::real d, a, b;      // kind 0/3: d, 1/h, 1/S; kind 2: -, w0, w1
-    typename Prec<MODE>::real alpha, e;
-    uint32_t off;                           // first table entry of the node's key
-    int16_t lo, npts;
-    uint8_t kind, woff;                     // kind 3: raw W_p values kept in the setup thread's row
-    uint16_t src;                           //   of the weight scratch, from column woff
+    typename Prec<MODE>::real b;
+    int lo, npts;
+    bool lng;
 };
 
-constexpr int MAXW = 12;                    // W_p values kept per node (longer supports recompute)
+// The accepted nodes that one warp spreads together (32 at most), in shared
+// memory: kernel values in a column per set-up lane (conflict-free for lanes
+// that read different nodes at the same point), the rest by the node's rank
+// among the nodes with work.
+template <int MODE>
+struct __align__(16) NodeBatch {
+    using real = typename Prec<MODE>::real;
+    real w[MAXW<MODE>][32];
+    uint2 key[32];                          // {first table entry less first (node, ray) pair, points packed}
+    real a[32], b[32];                      // alpha, weight factor (FP64 form: alpha x b / TW, -)
+    real e[32];                             // e (FP64 form: e x b / TW)
+    real eps[32], w1[32];                   // eps and the share of its second point (W_f,3)
+};
+// packing of a node's points: lo (7 bits), npts (8), set-up lane (5), first
+// point of eps (7), flags
+constexpr uint32_t PK_EPS = 1u << 27, PK_LONG = 1u << 28;
 
 // r_i of Eq. 4: in FP32 from its index, i^2 times a power of two (exact, no
 // load); in FP64 from the table (an FP64 multiply costs more than the load)
@@ -357,17 +386,6 @@ template <typename T>
 __device__ __forceinline__ T radius_at(int i, T coef, const double* tab) {
     if constexpr (sizeof(T) == 8) return __ldg(tab + i);
     else return (T)(i * i) * coef;
-}
-
-template <int MODE>
-__device__ __forceinline__ typename Prec<MODE>::real spread_weight(const RadialSpread<MODE>& n, int j,
-                                                                 typename Prec<MODE>::real rcoef, const double* rtab,
-                                                                 const typename Prec<MODE>::real* wts, int gauss) {
-    using real = typename Prec<MODE>::real;
-    if (n.kind == 3) return wts[n.src * MAXW + n.woff + j] * n.b;
-    if (n.kind == 0) return radial_w<real>(fabs(radius_at<real>(n.lo + j, rcoef, rtab) - n.d), n.a, gauss) * n.b;
-    if (n.kind == 1) return real(1);
-    return j == 0 ? n.a : n.b;
 }
 
 // W_p normalisation of an accepted node: the support of the kernel on the
@@ -378,60 +396,66 @@ __device__ __forceinline__ typename Prec<MODE>::real spread_weight(const RadialS
 // split) -- is not settled in FP32; radial_setup_exact then takes it in FP64.
 template <int MODE>
 __device__ __forceinline__ bool radial_setup(const WalkArgs& a, RadialSpread<MODE>& n, typename Prec<MODE>::real d,
-                                             int s, typename Prec<MODE>::real* wrow, int gauss, float dtol) {
+                                             int s, typename Prec<MODE>::real* wcol, int gauss, float dtol) {
     using real = typename Prec<MODE>::real;
     const int nr = a.nr;
     const real rc = (MODE == 0) ? (real)a.r_coef : (real)a.r_coeff;
-    n.d = d;
+    n.b = real(1); n.lng = false;
     const real rlast = radius_at<real>(nr - 1, rc, a.r);
     if (d >= rlast) {
-        n.kind = 1; n.lo = (int16_t)(nr - 1); n.npts = 1; n.a = real(1); n.b = real(1);
+        n.lo = nr - 1; n.npts = 1; wcol[0] = real(1);
         return MODE != 0 && (float)d - dtol < (float)rlast;
     }
     if (MODE != 0 && (float)d + dtol >= (float)rlast) return true;
     const real h = (real)s, inv_h = real(1) / h;
     const real hpar = gauss ? h : inv_h;
     const real reach = real(0.8661) * h + (real)dtol;
-    // a point whose kernel argument lies within xtol of sqrt3/2 may fall on
-    // the other side of the support's edge in FP64
-    const float xtol = MODE != 0 ? 2.f * (dtol + U32 * (2.f * (float)d + (float)reach)) * (float)inv_h + 4.f * U32
-                                 : 0.f;
-    int n_sure = 0;
-    bool near_edge = false;
     const real dlo = d > reach ? d - reach : real(0);
     // floor / ceil of the support's index bounds (i = eta sqrt(2 r), Eq. 4),
-    // in FP32 in both forms: an error below one index only widens the range
-    // by a point, and the weights themselves are computed in the form's
-    // precision (an FP64 square root costs a dozen FP64-pipe instructions)
-    const int lo = max((int)floorf((float)a.eta * sqrtf(2.f * (float)dlo)), 0);
-    const int hi = min((int)ceilf((float)a.eta * sqrtf(2.f * (float)(d + reach))), nr - 1);
+    // from approximate FP32 roots in both forms and a margin above their
+    // error: it only widens the range by a point whose weight is zero, and
+    // the weights themselves are computed in the form's precision
+    const float el = 2.f * (float)dlo, eh = 2.f * (float)(d + reach);
+    const int lo = max((int)((float)a.eta * (el * rsqrtf(fmaxf(el, 1e-30f))) - 1e-3f), 0);
+    const int hi = min((int)((float)a.eta * (eh * rsqrtf(eh)) + 1.001f), nr - 1);
     real S = real(0);
-    int first = hi + 1, last = lo - 1;
-    const bool keep = MODE == 0 && hi - lo + 1 <= MAXW;
-    for (int i = lo; i <= hi; ++i) {
-        const real dist = fabs(radius_at<real>(i, rc, a.r) - d);
+    int cnt = 0, last = lo - 1;
+    real near = real(1e30);                 // the closest point
+    real* col = wcol;
+    float fi = (float)lo;
+    for (int i = lo; i <= hi; ++i, fi += 1.f) {
+        const real ri = MODE == 0 ? radius_at<real>(i, rc, a.r) : (real)(fi * fi) * rc;
+        const real dist = fabs(ri - d);
         const real w = radial_w<real>(dist, hpar, gauss);
-        if (keep) wrow[i - lo] = w;
-        if (w > real(0)) { S += w; first = min(first, i); last = i; }
-        if (MODE != 0) {
-            const bool ne = fabsf((float)(dist * inv_h) - (float)S3H_D) <= xtol;
-            near_edge |= ne;
-            n_sure += (w > real(0) && !ne) ? 1 : 0;
+        if (MODE != 0) near = fmin(near, dist);
+        if (w > real(0)) {                  // the support is one run of points
+            S += w;
+            last = i;
+            if (cnt < MAXW<MODE>) *col = w;
+            col += 32;
+            ++cnt;
         }
     }
-    if (MODE != 0 && near_edge && n_sure == 0) return true;
-    if (S > real(0)) {
-        n.kind = keep ? 3 : 0; n.woff = (uint8_t)(first - lo);
-        n.lo = (int16_t)first; n.npts = (int16_t)(last - first + 1); n.a = hpar; n.b = real(1) / S;
+    if (MODE != 0) {
+        // a point whose kernel argument lies within xtol of sqrt3/2 may fall
+        // on the other side of the support's edge in FP64; that matters when
+        // no point is surely inside, i.e. when the closest one is not
+        const float xtol = 2.f * (dtol + U32 * (2.f * (float)d + (float)reach)) * (float)inv_h + 4.f * U32;
+        const float x = (float)(near * inv_h) - (float)S3H_D;
+        if (!(x < -xtol) && x <= xtol) return true;
+    }
+    if (cnt > 0) {
+        n.lo = last - cnt + 1; n.npts = cnt; n.b = real(1) / S;
+        if (cnt > MAXW<MODE>) { n.lng = true; wcol[0] = d; wcol[32] = hpar; }
         return false;
     }
     int i = min(max((int)floorf((float)a.eta * sqrtf(2.f * (float)d)), 0), nr - 2);   // a guess, corrected below
     while (i + 1 < nr - 1 && radius_at<real>(i + 1, rc, a.r) <= d) ++i;
     while (i > 0 && radius_at<real>(i, rc, a.r) > d) --i;
     const real ra = radius_at<real>(i, rc, a.r), rb = radius_at<real>(i + 1, rc, a.r);
-    n.kind = 2; n.lo = (int16_t)i; n.npts = 2;
-    n.a = (rb - d) / (rb - ra);
-    n.b = (d - ra) / (rb - ra);
+    n.lo = i; n.npts = 2;
+    wcol[0] = (rb - d) / (rb - ra);
+    wcol[32] = (d - ra) / (rb - ra);
     return false;
 }
 
@@ -457,11 +481,12 @@ __device__ __forceinline__ int bracket_d(const double* r, int nr, int eta, doubl
 // none), so the weights are stored explicitly: one point (weight 1), two
 // consecutive points, or the linear split between the points bracketing d.
 template <int MODE>
-__device__ void radial_setup_exact(const WalkArgs& a, RadialSpread<MODE>& n, double d, int s, int gauss) {
+__device__ void radial_setup_exact(const WalkArgs& a, RadialSpread<MODE>& n, double d, int s,
+                                   typename Prec<MODE>::real* wcol, int gauss) {
     const int nr = a.nr;
-    n.d = (float)d;
+    n.b = 1.f; n.lng = false;
     if (d >= __ldg(a.r + nr - 1)) {
-        n.kind = 1; n.lo = (int16_t)(nr - 1); n.npts = 1; n.a = 1.f; n.b = 1.f;
+        n.lo = nr - 1; n.npts = 1; wcol[0] = 1.f;
         return;
     }
     const double h = (double)s, inv_h = 1.0 / h, hpar = gauss ? h : inv_h;
@@ -478,17 +503,18 @@ __device__ void radial_setup_exact(const WalkArgs& a, RadialSpread<MODE>& n, dou
             ++cnt;
         }
     }
-    if (cnt == 1) { n.kind = 1; n.lo = (int16_t)first; n.npts = 1; n.a = 1.f; n.b = 1.f; return; }
-    if (cnt == 2) { n.kind = 2; n.lo = (int16_t)first; n.npts = 2; n.a = (float)(w0 / S); n.b = (float)(w1 / S); return; }
+    if (cnt == 1) { n.lo = first; n.npts = 1; wcol[0] = 1.f; return; }
+    if (cnt == 2) { n.lo = first; n.npts = 2; wcol[0] = (float)(w0 / S); wcol[32] = (float)(w1 / S); return; }
     if (cnt > 2) {                          // not reached (FP32 saw no point well inside); FP32 weights
-        n.kind = 0; n.lo = (int16_t)first; n.npts = (int16_t)cnt; n.a = (float)hpar; n.b = (float)(1.0 / S);
+        n.lo = first; n.npts = cnt; n.lng = true; n.b = (float)(1.0 / S);
+        wcol[0] = (float)d; wcol[32] = (float)hpar;
         return;
     }
     const int i = bracket_d(a.r, nr, a.eta, d);
     const double ra = __ldg(a.r + i), rb = __ldg(a.r + i + 1);
-    n.kind = 2; n.lo = (int16_t)i; n.npts = 2;
-    n.a = (float)((rb - d) / (rb - ra));
-    n.b = (float)((d - ra) / (rb - ra));
+    n.lo = i; n.npts = 2;
+    wcol[0] = (float)((rb - d) / (rb - ra));
+    wcol[32] = (float)((d - ra) / (rb - ra));
 }
 
 // two-point W_f,3: the sum and the flux at r = 0 exact
@@ -594,48 +620,25 @@ __device__ __forceinline__ void deposit_eps_variant(const WalkArgs& a, double* b
     }
 }
 
-// Deposit of an emitting node's eps (App. A.3).  Default W_f,3: two points
-// r_i <= d < r_{i+1} keeping the sum and the flux at the target exact (a
-// continuous function of d).  The other kernels take their FP64 distance
-// dvar (in the FP32 forms, from the FP64 tree: their choices jump).
-// Emitting nodes are few (they contain a source), so the accepting thread
-// does it alone.
-template <int MODE, bool VAR>
-__device__ void deposit_eps(const WalkArgs& a, double* bins_eps, uint32_t off, int ne,
-                            typename Prec<MODE>::real d, typename Prec<MODE>::real eps, float scale, int s_edge,
-                            double dvar) {
+// The default eps kernel W_f,3 (App. A.3): two points r_i <= d < r_{i+1}
+// keeping the sum and the flux at the target exact (a continuous function of
+// d).  Returns i; the second point's share in w1, the first's is 1 - w1.
+template <int MODE>
+__device__ __forceinline__ int eps_split(const WalkArgs& a, typename Prec<MODE>::real d, typename Prec<MODE>::real& w1) {
     using real = typename Prec<MODE>::real;
     const int nr = a.nr;
-    if (VAR && a.kern_e != TR_EPS_WF3) {
-        deposit_eps_variant<MODE>(a, bins_eps, off, ne, dvar, eps, scale, s_edge);
-        return;
-    }
     const real* r = (MODE == 0) ? reinterpret_cast<const real*>(a.r) : reinterpret_cast<const real*>(a.rf);
-    int i;
-    real w0, w1;
-    if (d >= r[nr - 1]) {
-        i = nr - 2; w0 = real(0); w1 = real(1);
-    } else {
-        i = min(max((int)floorf((float)a.eta * sqrtf(2.f * (float)d)), 0), nr - 2);   // a guess, corrected below
-        while (i + 1 < nr - 1 && r[i + 1] <= d) ++i;
-        while (i > 0 && r[i] > d) --i;
-        if (i == 0) {
-            w0 = real(0); w1 = real(1);
-        } else {
-            const real ri = r[i], rj = r[i + 1];
-            const real ia = real(1) / (ri * ri), ib = real(1) / (rj * rj), it = real(1) / (d * d);
-            w1 = (ia - it) / (ia - ib);
-            w0 = real(1) - w1;
-        }
+    w1 = real(1);
+    if (d >= r[nr - 1]) return nr - 2;
+    int i = min(max((int)floorf((float)a.eta * sqrtf(2.f * (float)d)), 0), nr - 2);   // a guess, corrected below
+    while (i + 1 < nr - 1 && r[i + 1] <= d) ++i;
+    while (i > 0 && r[i] > d) --i;
+    if (i > 0) {
+        const real ri = r[i], rj = r[i + 1];
+        const real ia = real(1) / (ri * ri), ib = real(1) / (rj * rj), it = real(1) / (d * d);
+        w1 = (ia - it) / (ia - ib);
     }
-    const real inv_m3 = real(1.0) / real(TW);
-    for (int k = 0; k < ne; ++k) {
-        const uint32_t en = __ldg(a.tent + off + k);
-        const int b = (int)(en >> 16) * nr + i;
-        const real wk = (real)(en & 0xffffu) * inv_m3;
-        if (w0 != real(0)) bin_atomic_add<MODE>(bins_eps + b, wk * w0 * eps, scale);
-        if (w1 != real(0)) bin_atomic_add<MODE>(bins_eps + b + 1, wk * w1 * eps, scale);
-    }
+    return i;
 }
 
 // 1/a in FP64 by the Newton-Raphson iteration y <- y + y (1 - a y), seeded with
@@ -689,7 +692,7 @@ __device__ __forceinline__ bool positive(double x) { return __double_as_longlong
 constexpr uint64_t EVEN_BITS = 0x5555555555555555ull;   // bits j with j % 2 == 0
 
 template <int MODE>
-__device__ double sweep_ray(const WalkArgs& a, const double* ba, double* be, const double* bee, const Scales& sc,
+__device__ __forceinline__ double sweep_ray(const WalkArgs& a, const double* ba, double* be, const double* bee, const Scales& sc,
                             int gl, unsigned gmask) {
     const int nr = a.nr;
     uint64_t m0 = 0, m1 = 0;
@@ -808,7 +811,7 @@ __device__ __forceinline__ float phi_f(const float2 E, const float2 Lr) {  // E 
 constexpr int SG = 2;
 constexpr uint64_t SG_PATTERN = 0x5555555555555555ull;   // bits j with j % 2 == 0
 
-__device__ double sweep_ray_group(const WalkArgs& a, const double* ba, double* be, const double* bee,
+__device__ __forceinline__ double sweep_ray_group(const WalkArgs& a, const double* ba, double* be, const double* bee,
                                   const Scales& sc, int gl, unsigned gmask) {
     const int nr = a.nr;
     uint64_t m0 = 0, m1 = 0;
@@ -975,7 +978,7 @@ __device__ __forceinline__ void rank_rays(const WalkArgs& a, const double* bins_
 // ray with one point and no e has zeta_s = zeta_d = 1, R_ij = A_i G_ij.
 // Each group's first lane returns its ray's F_0 (FP64) in the sum.
 template <int NT>
-__device__ double sweep_groups(const WalkArgs& a, const double* bins_a, const double* bins_eps, const double* bins_e,
+__device__ __forceinline__ double sweep_groups(const WalkArgs& a, const double* bins_a, const double* bins_eps, const double* bins_e,
                                const Scales& sc, const unsigned char* scratch) {
     const int npix = a.npix, nr = a.nr, lane = threadIdx.x & 31;
     const uint16_t* order = reinterpret_cast<const uint16_t*>(scratch);
@@ -1135,23 +1138,23 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // pops NT/8 opened nodes and evaluates their NT children, one per thread.
 // Per-thread walk counters go to the job's counters (one atomic per warp).
 struct WalkCounters {
-    unsigned long long vis = 0, acc = 0, ent = 0;
+    unsigned vis = 0, acc = 0, ent = 0;     // (flushed before they can wrap)
     unsigned fb_mac = 0, fb_dep = 0;        // FP32 forms: decisions re-taken in FP64
 };
 
 __device__ __forceinline__ void flush_counters(const WalkArgs& a, WalkCounters& c) {
-    unsigned long long fm = c.fb_mac, fd = c.fb_dep;
+    unsigned long long fm = c.fb_mac, fd = c.fb_dep, vis = c.vis, acc = c.acc, ent = c.ent;
     for (int o = 16; o > 0; o >>= 1) {
-        c.vis += __shfl_xor_sync(FULL, c.vis, o);
-        c.acc += __shfl_xor_sync(FULL, c.acc, o);
-        c.ent += __shfl_xor_sync(FULL, c.ent, o);
+        vis += __shfl_xor_sync(FULL, vis, o);
+        acc += __shfl_xor_sync(FULL, acc, o);
+        ent += __shfl_xor_sync(FULL, ent, o);
         fm += __shfl_xor_sync(FULL, fm, o);
         fd += __shfl_xor_sync(FULL, fd, o);
     }
     if ((threadIdx.x & 31) == 0) {
-        atomicAdd(a.stats + 0, c.vis);
-        atomicAdd(a.stats + 1, c.acc);
-        atomicAdd(a.stats + 2, c.ent);
+        atomicAdd(a.stats + 0, vis);
+        atomicAdd(a.stats + 1, acc);
+        atomicAdd(a.stats + 2, ent);
         if (fm) atomicAdd(a.stats + 3, fm);
         if (fd) atomicAdd(a.stats + 4, fd);
     }
@@ -1169,19 +1172,260 @@ __device__ __forceinline__ void flush_counters(const WalkArgs& a, WalkCounters& 
 // accepted ids; OUT_CD column-density maps (no radial points, no sweep).
 constexpr int OUT_FUSED = 0, OUT_DUMP = 1, OUT_CD = 2;
 
-// Column-density map deposit of an accepted node (cdMaps): each table entry
-// (ray k, volume fraction w_k) adds w_k m / (Omega d^2).
+// A target cell: its corner and edge (finest cells) and centre.
 template <int MODE>
-__device__ __forceinline__ void deposit_cd(const WalkArgs& a, double* bins, uint32_t off, int ne,
-                                           typename Prec<MODE>::real m, typename Prec<MODE>::real d) {
-    const double md = (double)m / (a.cd_omega * ((double)d * (double)d));
-    const double inv_m3 = 1.0 / (double)TW;
-    for (int k = 0; k < ne; ++k) {
-        const uint32_t en = __ldg(a.tent + off + k);
-        atomicAdd(bins + (en >> 16), ((double)(en & 0xffffu) * inv_m3) * md);
+struct Target {
+    typename Prec<MODE>::real px, py, pz;
+    int tx, ty, tz, ts;
+};
+
+// Where a node lies as seen from the target, in the copy that the boundary
+// puts there: offset o = 2 (node centre - target centre) in half cells, and
+// the squared distance of its centre of mass (FP32 forms: within B of the
+// FP64 value).
+template <int MODE>
+struct NodeView {
+    typename Prec<MODE>::real qx, qy, qz, d2;
+    float B;
+    int ox, oy, oz;
+};
+
+template <int MODE, bool VAR>
+__device__ __forceinline__ NodeView<MODE> view_node(const WalkArgs& a, const Target<MODE>& t, int img, int cx, int cy,
+                                                    int cz, int s, const typename Prec<MODE>::real* cm, float kap) {
+    using real = typename Prec<MODE>::real;
+    NodeView<MODE> v;
+    v.ox = 2 * cx + s - 2 * t.tx - t.ts; v.oy = 2 * cy + s - 2 * t.ty - t.ts; v.oz = 2 * cz + s - 2 * t.tz - t.ts;
+    v.qx = t.px; v.qy = t.py; v.qz = t.pz;
+    if (VAR && a.bc != TR_BC_ISOLATED) {
+        bc_frame<real>(a.bc, img & 1, a.N, 2 * cx + s, 2 * t.tx + t.ts, t.px, v.ox, v.qx);
+        bc_frame<real>(a.bc, (img >> 1) & 1, a.N, 2 * cy + s, 2 * t.ty + t.ts, t.py, v.oy, v.qy);
+        bc_frame<real>(a.bc, (img >> 2) & 1, a.N, 2 * cz + s, 2 * t.tz + t.ts, t.pz, v.oz, v.qz);
     }
+    if constexpr (MODE == 0) {
+        v.d2 = dist2(v.qx, v.qy, v.qz, cm);
+        v.B = 0.f;
+    } else {
+        // centre of mass - target = o/2 + offset (a mirror image of the corner
+        // of symmetry mirrors the offset too)
+        const bool mir = VAR && a.bc == TR_BC_CORNER;
+        const float ex = fmaf(0.5f, (float)v.ox, (mir && (img & 1)) ? -cm[0] : cm[0]);
+        const float ey = fmaf(0.5f, (float)v.oy, (mir && (img & 2)) ? -cm[1] : cm[1]);
+        const float ez = fmaf(0.5f, (float)v.oz, (mir && (img & 4)) ? -cm[2] : cm[2]);
+        v.d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+        v.B = d2_err_bound(v.d2, kap * (float)s);
+    }
+    return v;
 }
 
+struct Bins {
+    double *a, *eps, *e;                    // e: only with e_prev
+};
+
+// Map and spread up to 32 accepted nodes onto the target's rays, by one warp
+// and without a barrier of the CTA.  First a lane per node: its table key,
+// its ray entries and its radial weights.  Then a lane per (node, ray) pair,
+// the pairs of all 32 nodes laid end to end: a lane finds its node from the
+// bit mask of the pairs that start a node, loads the table entry a round
+// ahead, and adds to the node's points on that ray.  Both halves keep the
+// lanes full, which a thread that evaluates a node and then spreads it
+// cannot: at theta = 0.5 three quarters of the evaluated nodes are accepted,
+// and a node has 1 to 20 rays and 1 to 10 points.
+template <int MODE, int OUT, bool VAR>
+__device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>& nb, uint32_t entry, bool have, int img,
+                                             const Target<MODE>& t, const Bins& bins, const Scales& sc, float kap,
+                                             WalkCounters& cnt) {
+    using real = typename Prec<MODE>::real;
+    constexpr bool CD = OUT == OUT_CD;
+    const int lane = threadIdx.x & 31, nr = a.nr;
+    const bool use_e = a.use_e != 0;
+    const uint32_t* const tent = a.tent;
+    int ne = 0, eps_i = 0;
+    uint32_t off = 0;
+    RadialSpread<MODE> n;
+    n.b = real(1); n.lo = 0; n.npts = 0; n.lng = false;
+    real alpha = real(0), e = real(0), eps = real(0), w1 = real(0);
+    double md = 0.0;
+    if (have) {
+        const int lev = (int)(entry >> 27);
+        const uint32_t mort = entry & 0x7ffffffu;
+        const int s = a.N >> lev;
+        const int cx = (int)compact3(mort) * s, cy = (int)compact3(mort >> 1) * s, cz = (int)compact3(mort >> 2) * s;
+        const int64_t nid = level_offset(lev) + mort;
+        real cm[3], m, qv[3], mion;
+        load_node<MODE>(a.nodes, nid, cm, m, qv, mion);
+        const NodeView<MODE> v = view_node<MODE, VAR>(a, t, img, cx, cy, cz, s, cm, kap);
+        const real d = sqrt(v.d2);
+        if (CD) {
+            const uint2 hd = __ldg(a.hdr + table_key(v.ox, v.oy, v.oz, s));
+            off = hd.x; ne = (int)hd.y;
+            md = (double)m / (a.cd_omega * ((double)d * (double)d));
+            cnt.ent += ne;
+        } else {
+            // FP32 forms: |d - d64| <= dtol; the choices that jump with d and
+            // lie closer than that are taken on d64
+            const float dtol = MODE != 0 ? __fdividef(v.B, (float)d) + 4.f * U32 * (float)d : 0.f;
+            double d64 = -1.0;
+            auto exact_d = [&]() -> double {
+                if (d64 < 0.0) { d64 = sqrt(exact_d2(a, nid, v.qx, v.qy, v.qz)); ++cnt.fb_dep; }
+                return d64;
+            };
+            bool in_reach;
+            if constexpr (MODE == 0) {
+                in_reach = d <= a.lray;
+            } else {
+                if ((float)d + dtol < a.lrayf * (1.f - 2.f * U32)) in_reach = true;
+                else if ((float)d - dtol > a.lrayf * (1.f + 2.f * U32)) in_reach = false;
+                else in_reach = exact_d() <= a.lray;
+            }
+            if (in_reach) {
+                const uint2 hd = __ldg(a.hdr + table_key(v.ox, v.oy, v.oz, s));
+                off = hd.x; ne = (int)hd.y;
+                cnt.ent += ne;
+                if (qv[1] != real(0)) {
+                    if (VAR && a.kern_e != TR_EPS_WF3) {
+                        const double dvar = MODE != 0 ? exact_d() : (double)d;
+                        deposit_eps_variant<MODE>(a, bins.eps, off, ne, dvar, qv[1], sc.eps, s);
+                    } else {
+                        eps = qv[1];
+                        eps_i = eps_split<MODE>(a, d, w1);
+                    }
+                }
+                if (qv[0] != real(0) || (a.use_e && qv[2] != real(0))) {
+                    const int gauss = VAR ? a.kern_a : 0;
+                    if (radial_setup<MODE>(a, n, d, s, &nb.w[0][lane], gauss, dtol)) {
+                        if constexpr (MODE != 0) radial_setup_exact<MODE>(a, n, exact_d(), s, &nb.w[0][lane], gauss);
+                    }
+                    alpha = qv[0];
+                    e = a.use_e ? qv[2] : real(0);
+                }
+            }
+        }
+    }
+    // the batch's (node, ray) pairs, end to end
+    const bool act = ne > 0 && (CD || n.npts > 0 || eps != real(0));
+    if (!act) ne = 0;
+    int incl = ne;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const int total = __shfl_sync(FULL, incl, 31), start = incl - ne;
+    const unsigned am = __ballot_sync(FULL, act), lt = (1u << lane) - 1u;
+    if (act) {
+        const int k = __popc(am & lt);
+        nb.key[k] = make_uint2(off - (uint32_t)start,
+                               (uint32_t)n.lo | ((uint32_t)n.npts << 7) | ((uint32_t)lane << 15) |
+                                   ((uint32_t)eps_i << 20) | (eps != real(0) ? PK_EPS : 0u) | (n.lng ? PK_LONG : 0u));
+        if constexpr (CD) {
+            reinterpret_cast<double*>(&nb.w[0][0])[k] = md;
+        } else if constexpr (MODE == 0) {
+            const double f = n.b * (1.0 / TW);
+            nb.a[k] = alpha * f; nb.e[k] = e * f;
+            nb.eps[k] = eps; nb.w1[k] = w1;
+        } else {
+            nb.a[k] = alpha; nb.b[k] = n.b; nb.e[k] = e;
+            nb.eps[k] = eps; nb.w1[k] = w1;
+        }
+    }
+    __syncwarp();
+    int before = -1;                                         // nodes started before the round, less one
+    int k = 0;
+    uint32_t en = 0;
+    uint2 key = make_uint2(0u, 0u);
+    auto locate = [&](int base) {                            // the lane's node and table entry of round `base`
+        const unsigned m = __reduce_or_sync(FULL, act && (start >> 5) == (base >> 5) ? 1u << (start & 31) : 0u);
+        k = before + __popc(m & (lt | (1u << lane)));
+        before += __popc(m);
+        if (base + lane < total) {
+            key = nb.key[k];
+            en = __ldg(tent + (uint32_t)(key.x + (uint32_t)(base + lane)));
+        }
+    };
+    if (total > 0) locate(0);
+    for (int base = 0; base < total; base += 32) {
+        const int kc = k;
+        const uint32_t ec = en, pk = key.y;
+        if (base + 32 < total) locate(base + 32);
+        if (base + lane >= total) continue;
+        const int ray = (int)(ec >> 16);
+        if constexpr (CD) {
+            const double wk = (double)(ec & 0xffffu) * (1.0 / TW);
+            atomicAdd(bins.a + ray, wk * reinterpret_cast<const double*>(&nb.w[0][0])[kc]);
+            continue;
+        }
+        const int npts = (int)(pk >> 7) & 0xff, src = (int)(pk >> 15) & 31;
+        const int b0 = ray * nr + (int)(pk & 0x7fu);
+        const real* wc = &nb.w[0][src];
+        if constexpr (MODE == 0) {
+            const double c = (double)(ec & 0xffffu);
+            const double ca = c * nb.a[kc], ce = use_e ? c * nb.e[kc] : 0.0;
+            const double d = wc[0], hpar = wc[32];
+            for (int j = 0; j < npts; ++j) {
+                const double w = (pk & PK_LONG)
+                                     ? radial_w<double>(fabs(radius_at<double>((int)(pk & 0x7fu) + j, a.r_coef, a.r) - d), hpar, VAR ? a.kern_a : 0)
+                                     : wc[j * 32];
+                if (ca != 0.0) atomicAdd(bins.a + b0 + j, w * ca);
+                if (use_e && ce != 0.0) atomicAdd(bins.e + b0 + j, w * ce);
+            }
+        } else {
+            // ((W b) cnt) (alpha scale / TW): the scales are powers of two
+            const float c = (float)(ec & 0xffffu), b = nb.b[kc];
+            const float al = nb.a[kc] * (sc.a * (1.f / TW)), ee = use_e ? nb.e[kc] * (sc.e * (1.f / TW)) : 0.f;
+            double* ba = bins.a + b0;
+            double* be = bins.e + b0;
+            if (!(pk & PK_LONG)) {
+                for (int j = 0; j < npts; ++j) {
+                    const float w = wc[j * 32] * b * c;
+                    bin_add_units(ba + j, w * al);
+                    if (use_e) bin_add_units(be + j, w * ee);
+                }
+            } else {
+                const float d = wc[0], hpar = wc[32];
+                for (int j = 0; j < npts; ++j) {
+                    const float w = radial_w<float>(fabsf(radius_at<float>((int)(pk & 0x7fu) + j, a.r_coeff, a.r) - d),
+                                                    hpar, VAR ? a.kern_a : 0) * b * c;
+                    bin_add_units(ba + j, w * al);
+                    if (use_e) bin_add_units(be + j, w * ee);
+                }
+            }
+        }
+        if (pk & PK_EPS) {
+            const real wk = (real)(ec & 0xffffu) * (real(1) / TW);
+            const real ep = nb.eps[kc], s1 = nb.w1[kc], s0 = real(1) - s1;
+            double* be = bins.eps + ray * nr + ((int)(pk >> 20) & 0x7f);
+            if (s0 != real(0)) bin_atomic_add<MODE>(be, wk * s0 * ep, sc.eps);
+            if (s1 != real(0)) bin_atomic_add<MODE>(be + 1, wk * s1 * ep, sc.eps);
+        }
+    }
+    __syncwarp();                                            // the batch read before the next one is written
+}
+
+// The list of accepted nodes waiting to be spread: 4 NT entries, spread when
+// a step could overflow it (three full batches of 32 per warp) and at the end.
+template <int NT> constexpr int acc_cap() { return 4 * NT; }
+
+// Opened nodes waiting in a target's ring buffer.  It never holds more than
+// the target's opened nodes (a few hundred at theta = 0.5); overflow is
+// detected and reported, never written past.  While at most FIFO_MAX wait,
+// the oldest are taken first, so that the list fills level by level and a
+// batch of 32 accepted nodes has like numbers of points and rays; beyond
+// that the newest (a depth-first walk, which bounds the buffer: 64 waiting
+// nodes and one step's pushes are what it holds at the same depth).
+constexpr int STACK_CAP = 512;
+constexpr int FIFO_MAX = 64;
+
+// A CTA of NT threads per target.  Walk step: take NT/8 opened nodes from the
+// shared buffer, evaluate their NT children, one per thread; opened children
+// go back into the buffer, accepted ones with something to map to a list.  When
+// the list is full, and at the end, the warps spread it (spread_nodes), 32
+// nodes a warp at a time, so that two barriers a step only separate short,
+// even work.  Bound by instruction issue and latency at 20 warps per SM (33
+// KB of bins per target); DRAM carries the tree once.  Setting up and
+// spreading the nodes of each step as they were accepted, as this walk did
+// before, left a third of the lanes idle and took turbulent128 from 217 to
+// 328 ms in the double-FP32 form (99 k to 62 k warp instructions per target
+// in the headline form).
 template <int MODE, int OUT, int NT, bool VAR>
 __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, const int64_t* __restrict__ job_end,
                                           int n_jobs, unsigned int* counter) {
@@ -1189,36 +1433,28 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
     constexpr int NW = NT / 32, P = NT / 8;
     constexpr bool DUMP = OUT == OUT_DUMP, CD = OUT == OUT_CD;
     extern __shared__ __align__(16) unsigned char smem[];
-    // per step: stack pushes, and spread nodes (high word) with their
-    // (node, ray) pairs (low word), reserved by one atomic per warp; two
-    // sets, by step parity, so that a set is cleared a step after its use
-    __shared__ int s_push[2];
-    __shared__ unsigned long long s_spread[2];
+    // per step: stack pushes (low half) and list entries (high half),
+    // reserved by one atomic per warp; two sets, by step parity, so that a
+    // set is cleared a step after its use
+    __shared__ unsigned s_cnt[2];
     __shared__ int s_over;
     __shared__ double s_red[NW];
     __shared__ unsigned int s_q;
     __shared__ int s_j;
     __shared__ int s_nacc;
     __shared__ __align__(16) WalkArgs s_a;                       // the current job
-    __shared__ RadialSpread<MODE> s_node[NT];                    // the step's nodes to spread
-    static_assert(sizeof(RadialSpread<MODE>) * NT >= sweep_scratch_bytes(MAX_NPIX), "sweep scratch in s_node");
-    __shared__ int s_pair0[NT + 1];                              // their first (node, ray) pair
-    // W_p values kept by the setup threads: the FP64 form saves recomputing
-    // them in FP64; in the FP32 form recomputing is cheaper than the shared
-    // memory (occupancy) they would take
-    __shared__ real s_w[MODE == 0 ? NT * MAXW : 1];
+    __shared__ NodeBatch<MODE> s_nb[NW];
+    static_assert(sizeof(NodeBatch<MODE>) * NW >= sweep_scratch_bytes(MAX_NPIX), "sweep scratch in s_nb");
+    __shared__ uint32_t s_acc[acc_cap<NT>()];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const WalkArgs& a = s_a;
     const unsigned lanemask_lt = (1u << lane) - 1u;
-    const real inv_m3 = real(1.0) / real(TW);
     const int64_t total = job_end[n_jobs - 1];
     WalkCounters cnt;                                        // per-thread counters
     float kap = 0.f;                                         // FP32 forms: the tree's kappa
     int cur = -1;
+    unsigned done = 0;                                       // targets since the counters were flushed
     int nr = 0, nbins = 0, nq = 2, N = 0, L = 0;
-    double *bins_a = nullptr, *bins_eps = nullptr, *bins_e = nullptr;
-    uint32_t* stack = nullptr;
-    real rcoef = real(0);
     Scales sc{1.f, 1.f, 1.f};
 
     for (;;) {
@@ -1233,8 +1469,8 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
         const int j = s_j;
         const int64_t qg = (int64_t)s_q;
         if (j < 0) break;
+        if (cur >= 0 && (j != cur || ++done >= 4096u)) { flush_counters(a, cnt); done = 0; }
         if (j != cur) {                                          // load the job (uniform over the CTA)
-            if (cur >= 0) flush_counters(a, cnt);
             __syncthreads();
             const int* src = reinterpret_cast<const int*>(jobs + j);
             int* dst = reinterpret_cast<int*>(&s_a);
@@ -1242,11 +1478,6 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
             __syncthreads();
             cur = j;
             nr = a.nr; nbins = CD ? a.npix : a.npix * nr; nq = CD ? 1 : (a.use_e ? 3 : 2); N = a.N; L = a.L;
-            bins_a = reinterpret_cast<double*>(smem);
-            bins_eps = bins_a + nbins;
-            bins_e = a.use_e ? bins_eps + nbins : nullptr;
-            stack = reinterpret_cast<uint32_t*>(bins_a + (size_t)nq * nbins);
-            rcoef = (MODE == 0) ? (real)a.r_coef : (real)a.r_coeff;
             if (MODE != 0) {                                     // fixed-point units from the root totals
                 real cm0[3], m0, q0[3], mi0;
                 load_node<MODE>(a.nodes, 0, cm0, m0, q0, mi0);
@@ -1256,6 +1487,11 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
                 kap = __ldg(a.kappa) * 1.000001f;
             }
         }
+        // derived from smem here, unconditionally, so that they stay shared-memory
+        // pointers to the compiler (a null on some path makes them generic)
+        double* const bins_a = reinterpret_cast<double*>(smem);
+        const Bins bins{bins_a, bins_a + nbins, bins_a + 2 * nbins};
+        uint32_t* const stack = reinterpret_cast<uint32_t*>(bins_a + nq * nbins);
         const int64_t q = qg - (j > 0 ? job_end[j - 1] : 0);    // index within the job
         if (a.targets) {                                         // caller's list: reject bad indices
             const int64_t c = a.targets[q];
@@ -1265,8 +1501,9 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
                 continue;
             }
         }
-        int tx, ty, tz;                                          // target corner (finest cells)
-        int ts = 1, tl = L;                                      // its edge and level
+        Target<MODE> t;
+        t.ts = 1;
+        int tl = L;                                              // the target's level
         int64_t cell;
         if (a.blk) {                                             // AMR: cell c of block b
             int b, lx, ly, lz;
@@ -1284,57 +1521,71 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
             }
             const int4 bm = __ldg(a.blk + b);
             tl = bm.x;
-            ts = N >> tl;
-            tx = (8 * bm.y + lx) * ts; ty = (8 * bm.z + ly) * ts; tz = (8 * bm.w + lz) * ts;
+            t.ts = N >> tl;
+            t.tx = (8 * bm.y + lx) * t.ts; t.ty = (8 * bm.z + ly) * t.ts; t.tz = (8 * bm.w + lz) * t.ts;
         } else if (a.targets) {
             cell = a.targets[q];
-            tx = (int)(cell % N); ty = (int)((cell / N) % N); tz = (int)(cell / ((int64_t)N * N));
+            t.tx = (int)(cell % N); t.ty = (int)((cell / N) % N); t.tz = (int)(cell / ((int64_t)N * N));
         } else {
             const uint32_t m = (uint32_t)(a.first + q);
-            tx = (int)compact3(m); ty = (int)compact3(m >> 1); tz = (int)compact3(m >> 2);
-            cell = ((int64_t)tz * N + ty) * N + tx;
+            t.tx = (int)compact3(m); t.ty = (int)compact3(m >> 1); t.tz = (int)compact3(m >> 2);
+            cell = ((int64_t)t.tz * N + t.ty) * N + t.tx;
         }
-        const real hts = real(0.5) * (real)ts;
-        const real px = (real)tx + hts, py = (real)ty + hts, pz = (real)tz + hts;
-        for (int b = tid; b < nq * nbins; b += NT) bins_a[b] = 0.0;
+        const real hts = real(0.5) * (real)t.ts;
+        t.px = (real)t.tx + hts; t.py = (real)t.ty + hts; t.pz = (real)t.tz + hts;
+        // (npix and so nbins is a multiple of 12)
+        for (int b = tid; b < nq * nbins / 2; b += NT) reinterpret_cast<double2*>(bins_a)[b] = make_double2(0.0, 0.0);
         if (tid == 0) {                                          // the root, opened
             stack[0] = 0u; s_nacc = 0;
-            s_push[0] = s_push[1] = 0; s_spread[0] = s_spread[1] = 0ull; s_over = 0;
+            s_cnt[0] = s_cnt[1] = 0u; s_over = 0;
         }
-        int top = 1, max_top = 1, par = 0;
+        int head = 0, top = 1, max_top = 1, par = 0, nl = 0;     // top: waiting nodes (from head on); nl: listed nodes
         bool overflow = false;
         __syncthreads();
+        // spread the last `take` listed nodes, 32 per warp at a time
+        auto spread_list = [&](int take, int img) {
+            for (int b = nl - take + wid * 32; b < nl; b += NT) {
+                const bool have = b + lane < nl;
+                spread_nodes<MODE, OUT, VAR>(a, s_nb[wid], have ? s_acc[b + lane] : 0u, have, img, t, bins, sc, kap, cnt);
+            }
+            nl -= take;
+        };
         // corner of symmetry: the original and its 7 mirror images (bit k of
         // img mirrors axis k through the low corner), all onto the same rays
         const int n_img = (VAR && a.bc == TR_BC_CORNER) ? 8 : 1;
         for (int img = 0; img < n_img && !overflow; ++img) {
         if (img > 0) {
-            if (tid == 0) stack[0] = ROOT_EVAL;
+            if (tid == 0) stack[head & (STACK_CAP - 1)] = ROOT_EVAL;
             top = 1;
-            __syncthreads();                                     // the image's root visible
+            __syncthreads();                                     // the image's root visible, the list read
         }
-        while (top > 0) {
+        for (;;) {
+            if (top == 0 || nl + NT > acc_cap<NT>()) {           // the walk's end, or a full list: full batches
+                spread_list(top == 0 ? nl : nl / NT * NT, img);
+                if (top == 0) break;
+            }
             const int np = min(P, top);
             const int pi = tid >> 3, c = tid & 7;
-            const uint32_t pe = (pi < np) ? stack[top - np + pi] : 0u;
-            __syncthreads();                                     // parents read before the pushes
+            const bool fifo = top <= FIFO_MAX;
+            const uint32_t pe = (pi < np) ? stack[(head + (fifo ? 0 : top - np) + pi) & (STACK_CAP - 1)] : 0u;
+            __syncthreads();                                     // parents and list read before they are overwritten
             top -= np;
+            if (fifo) head += np;
             int action = 0;                                      // 1 open, 2 accept
-            int lev = 0, ne = 0;
-            uint32_t mort = 0;
-            RadialSpread<MODE> node;
-            bool spread = false;
+            uint32_t ent = 0;                                    // the child as a stack or list entry
+            bool list = false;
             // ROOT_EVAL: the root itself is evaluated (a mirror image does not
             // contain the target, so its root is subject to the MACs)
             if (pi < np && (!VAR || pe != ROOT_EVAL || c == 0)) {
                 ++cnt.vis;
-                lev = (VAR && pe == ROOT_EVAL) ? 0 : (int)(pe >> 27) + 1;
-                mort = (VAR && pe == ROOT_EVAL) ? 0u : (((pe & 0x7ffffffu) << 3) | (uint32_t)c);
+                const int lev = (VAR && pe == ROOT_EVAL) ? 0 : (int)(pe >> 27) + 1;
+                const uint32_t mort = (VAR && pe == ROOT_EVAL) ? 0u : (((pe & 0x7ffffffu) << 3) | (uint32_t)c);
+                ent = ((uint32_t)lev << 27) | mort;
                 const int s = N >> lev;
                 const int cx = (int)compact3(mort) * s, cy = (int)compact3(mort >> 1) * s,
                           cz = (int)compact3(mort >> 2) * s;
-                const bool contains = img == 0 && (tx >= cx && tx < cx + s) && (ty >= cy && ty < cy + s) &&
-                                      (tz >= cz && tz < cz + s);
+                const bool contains = img == 0 && (t.tx >= cx && t.tx < cx + s) && (t.ty >= cy && t.ty < cy + s) &&
+                                      (t.tz >= cz && t.tz < cz + s);
                 const int64_t nid = level_offset(lev) + mort;
                 const bool leaf = a.flags ? (__ldg(a.flags + nid) == NODE_LEAF) : (lev == L);
                 if (contains) {
@@ -1342,219 +1593,58 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
                 } else {
                     real cm[3], m, qv[3], mion;
                     load_node<MODE>(a.nodes, nid, cm, m, qv, mion);
-                    // offset o = 2 (node centre - target centre) in half cells of the node
-                    // copy that the boundary puts next to the target, and the target
-                    // centre to measure that copy's distance from in the node's frame
-                    int ox = 2 * cx + s - 2 * tx - ts, oy = 2 * cy + s - 2 * ty - ts, oz = 2 * cz + s - 2 * tz - ts;
-                    real qx = px, qy = py, qz = pz;
-                    if (VAR && a.bc != TR_BC_ISOLATED) {
-                        bc_frame<real>(a.bc, img & 1, N, 2 * cx + s, 2 * tx + ts, px, ox, qx);
-                        bc_frame<real>(a.bc, (img >> 1) & 1, N, 2 * cy + s, 2 * ty + ts, py, oy, qy);
-                        bc_frame<real>(a.bc, (img >> 2) & 1, N, 2 * cz + s, 2 * tz + ts, pz, oz, qz);
-                    }
-                    real d2;
-                    float B = 0.f;                       // FP32 forms: bound on |d2 - d2 in FP64|
-                    if constexpr (MODE == 0) {
-                        d2 = dist2(qx, qy, qz, cm);
-                    } else {
-                        // centre of mass - target = o/2 + offset (a mirror image
-                        // of the corner of symmetry mirrors the offset too)
-                        const bool mir = VAR && a.bc == TR_BC_CORNER;
-                        const float ex = fmaf(0.5f, (float)ox, (mir && (img & 1)) ? -cm[0] : cm[0]);
-                        const float ey = fmaf(0.5f, (float)oy, (mir && (img & 2)) ? -cm[1] : cm[1]);
-                        const float ez = fmaf(0.5f, (float)oz, (mir && (img & 4)) ? -cm[2] : cm[2]);
-                        d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-                        B = d2_err_bound(d2, kap * (float)s);
-                    }
-                    const real h2 = (real)s * (real)s;
                     bool open = false;
                     if (!leaf) {
+                        const NodeView<MODE> v = view_node<MODE, VAR>(a, t, img, cx, cy, cz, s, cm, kap);
+                        const real h2 = (real)s * (real)s;
                         if constexpr (MODE == 0) {
-                            open = must_open(h2, d2, m, mion, qv[1], a);
+                            open = must_open(h2, v.d2, m, mion, qv[1], a);
                         } else {
-                            const int r = mac_f32(h2, d2, B, signbit(mion), qv[1] > 0.f, a);
+                            const int r = mac_f32(h2, v.d2, v.B, signbit(mion), qv[1] > 0.f, a);
                             if (r < 0) {
                                 ++cnt.fb_mac;
-                                open = must_open_exact((double)h2, exact_d2(a, nid, qx, qy, qz), signbit(mion),
+                                open = must_open_exact((double)h2, exact_d2(a, nid, v.qx, v.qy, v.qz), signbit(mion),
                                                        qv[1] > 0.f, a);
                             } else {
                                 open = r == 1;
                             }
                         }
                     }
-                    if (open) {
-                        action = 1;
-                    } else if (CD) {
-                        action = 2;
-                        if (m > real(0)) {
-                            const uint2 hd = __ldg(a.hdr + table_key(ox, oy, oz, s));
-                            cnt.ent += hd.y;
-                            deposit_cd<MODE>(a, bins_a, hd.x, (int)hd.y, m, sqrt(d2));
-                        }
-                    } else {
-                        action = 2;
-                        const real d = sqrt(d2);
-                        // FP32 forms: |d - d64| <= dtol; the choices that jump
-                        // with d and lie closer than that are taken on d64
-                        const float dtol = MODE != 0 ? B / (float)d + 4.f * U32 * (float)d : 0.f;
-                        double d64 = -1.0;
-                        auto exact_d = [&]() -> double {
-                            if (d64 < 0.0) { d64 = sqrt(exact_d2(a, nid, qx, qy, qz)); ++cnt.fb_dep; }
-                            return d64;
-                        };
-                        bool in_reach;
-                        if constexpr (MODE == 0) {
-                            in_reach = d <= a.lray;
-                        } else {
-                            if ((float)d + dtol < a.lrayf * (1.f - 2.f * U32)) in_reach = true;
-                            else if ((float)d - dtol > a.lrayf * (1.f + 2.f * U32)) in_reach = false;
-                            else in_reach = exact_d() <= a.lray;
-                        }
-                        const bool has_ae = qv[0] != real(0) || (a.use_e && qv[2] != real(0));
-                        if (in_reach && (has_ae || qv[1] != real(0))) {
-                            const int key = table_key(ox, oy, oz, s);
-                            const uint2 hd = __ldg(a.hdr + key);
-                            ne = (int)hd.y;
-                            cnt.ent += ne;
-                            if (qv[1] != real(0)) {
-                                const double dvar = (MODE != 0 && VAR && a.kern_e != TR_EPS_WF3) ? exact_d() : (double)d;
-                                deposit_eps<MODE, VAR>(a, bins_eps, hd.x, ne, d, qv[1], sc.eps, s, dvar);
-                            }
-                            if (has_ae && ne > 0) {
-                                const int gauss = VAR ? a.kern_a : 0;
-                                if (radial_setup<MODE>(a, node, d, s, s_w + tid * MAXW, gauss, dtol)) {
-                                    if constexpr (MODE != 0) radial_setup_exact<MODE>(a, node, exact_d(), s, gauss);
-                                }
-                                node.src = (uint16_t)tid;
-                                node.alpha = qv[0];
-                                node.e = a.use_e ? qv[2] : real(0);
-                                node.off = hd.x;
-                                spread = true;
-                            }
-                        }
-                    }
+                    action = open ? 1 : 2;
+                    list = !open && (CD ? m > real(0)
+                                        : (qv[0] != real(0) || qv[1] != real(0) || (a.use_e && qv[2] != real(0))));
                 }
             }
-            // stack slots of the pushes and spread-list slots of the nodes to
-            // spread: one shared atomic per warp reserves them (the order of
-            // the warps' blocks is immaterial: fixed-point or FP64 atomic
-            // deposits, accepted nodes a set)
+            // slots of the pushes and of the listed nodes: one shared atomic
+            // per warp reserves both (the order of the warps' blocks is
+            // immaterial: fixed-point or FP64 atomic deposits, accepted
+            // nodes a set)
             const unsigned om = __ballot_sync(FULL, action == 1);
-            const unsigned bm = __ballot_sync(FULL, spread);
-            // work items of this thread's node: (ray, point) triples (FP64) or rays (FP32)
-            int pc = spread ? (MODE == 0 ? ne * node.npts : ne) : 0;
-            int incl = pc;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int wpairs = __shfl_sync(FULL, incl, 31);      // the warp's pairs
-            int obase = 0;
-            unsigned long long nbp = 0ull;
-            if (lane == 0) {
-                if (om) obase = atomicAdd(&s_push[par], __popc(om));
-                if (bm) nbp = atomicAdd(&s_spread[par], ((unsigned long long)__popc(bm) << 32) |
-                                                          (unsigned long long)(unsigned)wpairs);
-            }
-            obase = __shfl_sync(FULL, obase, 0);
-            nbp = __shfl_sync(FULL, nbp, 0);
+            const unsigned bm = __ballot_sync(FULL, list);
+            unsigned base = 0;
+            if (lane == 0 && (om | bm)) base = atomicAdd(&s_cnt[par], ((unsigned)__popc(bm) << 16) | (unsigned)__popc(om));
+            base = __shfl_sync(FULL, base, 0);
             if (action == 1) {
-                const int slot = top + obase + __popc(om & lanemask_lt);
-                if (slot < a.stack_cap) stack[slot] = ((uint32_t)lev << 27) | mort;
+                const int slot = top + (int)(base & 0xffffu) + __popc(om & lanemask_lt);
+                if (slot < STACK_CAP) stack[(head + slot) & (STACK_CAP - 1)] = ent;
                 else s_over = 1;                                 // never written past
             }
-            if (spread) {
-                const int k = (int)(nbp >> 32) + __popc(bm & lanemask_lt);
-                s_node[k] = node;
-                s_pair0[k] = (int)(nbp & 0xffffffffull) + incl - pc;
-            }
+            if (list) s_acc[nl + (int)(base >> 16) + __popc(bm & lanemask_lt)] = ent;   // nl + NT <= acc_cap
             if (action == 2) {
                 ++cnt.acc;
                 if (DUMP) {
                     const int slot = atomicAdd(&s_nacc, 1);
-                    if (slot < a.acc_cap) a.ids_out[q * a.acc_cap + slot] = (int32_t)(level_offset(lev) + mort);
+                    if (slot < a.acc_cap) a.ids_out[q * a.acc_cap + slot] = (int32_t)(level_offset((int)(ent >> 27)) + (ent & 0x7ffffffu));
                 }
             }
-            __syncthreads();                                     // pushes and spread list visible
-            const int ototal = s_push[par];
-            const unsigned long long sp = s_spread[par];
-            const int ntotal = (int)(sp >> 32), ptotal = (int)(sp & 0xffffffffull);
+            __syncthreads();                                     // pushes and list visible
+            const unsigned added = s_cnt[par];
             overflow = s_over != 0;                              // same value in every thread
-            if (tid == 0) { s_push[par ^ 1] = 0; s_spread[par ^ 1] = 0ull; }   // read by all a step ago
+            if (tid == 0) s_cnt[par ^ 1] = 0u;                   // read by all a step ago
             par ^= 1;
             if (overflow) break;
-            // spread the step's nodes.  FP64 form: each thread takes a contiguous
-            // run of (node, table entry, radial point) triples, so that every
-            // thread makes about the same number of deposits.  FP32 form: runs of
-            // (node, table entry) pairs with the points in an inner loop (the
-            // bookkeeping of the triples costs more than the balance gains there).
-            if constexpr (MODE == 0) {
-                if (ptotal > 0) {
-                    const int chunk = (ptotal + NT - 1) / NT;
-                    const int p0 = tid * chunk, p1 = min(p0 + chunk, ptotal);
-                    if (p0 < p1) {
-                        int k = 0, hi = ntotal - 1;
-                        while (k < hi) {
-                            const int mid = (k + hi + 1) >> 1;
-                            if (s_pair0[mid] <= p0) k = mid; else hi = mid - 1;
-                        }
-                        RadialSpread<MODE> n = s_node[k];
-                        const int li = p0 - s_pair0[k];
-                        int e = li / n.npts, j = li - e * n.npts;
-                        int ne_k = ((k + 1 < ntotal ? s_pair0[k + 1] : ptotal) - s_pair0[k]) / n.npts;
-                        uint32_t en = __ldg(a.tent + n.off + e);
-                        int b0 = (int)(en >> 16) * nr + n.lo;
-                        real wk = (real)(en & 0xffffu) * inv_m3;
-                        for (int p = p0; p < p1; ++p) {
-                            const real w = spread_weight<MODE>(n, j, rcoef, a.r, s_w, VAR ? a.kern_a : 0) * wk;
-                            if (w != real(0)) {
-                                if (n.alpha != real(0)) bin_atomic_add<MODE>(bins_a + b0 + j, w * n.alpha, sc.a);
-                                if (a.use_e && n.e != real(0)) bin_atomic_add<MODE>(bins_e + b0 + j, w * n.e, sc.e);
-                            }
-                            if (++j == n.npts) {                     // next table entry, or next node
-                                j = 0;
-                                if (++e == ne_k) {
-                                    if (p + 1 >= p1) break;
-                                    ++k;
-                                    n = s_node[k];
-                                    e = 0;
-                                    ne_k = ((k + 1 < ntotal ? s_pair0[k + 1] : ptotal) - s_pair0[k]) / n.npts;
-                                }
-                                en = __ldg(a.tent + n.off + e);
-                                b0 = (int)(en >> 16) * nr + n.lo;
-                                wk = (real)(en & 0xffffu) * inv_m3;
-                            }
-                        }
-                    }
-                }
-            } else {
-                if (ptotal > 0) {
-                    const int chunk = (ptotal + NT - 1) / NT;
-                    const int p0 = tid * chunk, p1 = min(p0 + chunk, ptotal);
-                    if (p0 < p1) {
-                        int k = 0, hi = ntotal - 1;
-                        while (k < hi) {
-                            const int mid = (k + hi + 1) >> 1;
-                            if (s_pair0[mid] <= p0) k = mid; else hi = mid - 1;
-                        }
-                        RadialSpread<MODE> n = s_node[k];
-                        int kend = k + 1 < ntotal ? s_pair0[k + 1] : ptotal;
-                        for (int p = p0; p < p1; ++p) {
-                            if (p >= kend) { ++k; n = s_node[k]; kend = k + 1 < ntotal ? s_pair0[k + 1] : ptotal; }
-                            const uint32_t en = __ldg(a.tent + n.off + (p - s_pair0[k]));
-                            const int b0 = (int)(en >> 16) * nr + n.lo;
-                            const real wk = (real)(en & 0xffffu) * inv_m3;
-                            for (int j = 0; j < n.npts; ++j) {
-                                const real w = spread_weight<MODE>(n, j, rcoef, a.r, s_w, VAR ? a.kern_a : 0) * wk;
-                                if (w == real(0)) continue;
-                                if (n.alpha != real(0)) bin_atomic_add<MODE>(bins_a + b0 + j, w * n.alpha, sc.a);
-                                if (a.use_e && n.e != real(0)) bin_atomic_add<MODE>(bins_e + b0 + j, w * n.e, sc.e);
-                            }
-                        }
-                    }
-                }
-            }
-            top += ototal;
+            top += (int)(added & 0xffffu);
+            nl += (int)(added >> 16);
             max_top = max(max_top, top);
         }
         }                                                        // images
@@ -1566,14 +1656,14 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
                 continue;
             }
             double* out = a.cd_out + (size_t)(a.targets ? q : cell) * a.npix;
-            for (int k = tid; k < a.npix; k += NT) out[k] = bins_a[k] * a.cd_conv;
+            for (int k = tid; k < a.npix; k += NT) out[k] = bins.a[k] * a.cd_conv;
             continue;
         }
         // own emission of the target (Sec. 2.5 footnote: target sphere of
         // radius r_tp = half the cell edge)
         real cmt[3], mt, qt[3], miont;
-        load_node<MODE>(a.nodes, level_offset(tl) + morton3(tx / ts, ty / ts, tz / ts), cmt, mt, qt, miont);
-        const double r_tp2 = 0.25 * (double)ts * (double)ts;
+        load_node<MODE>(a.nodes, level_offset(tl) + morton3(t.tx / t.ts, t.ty / t.ts, t.tz / t.ts), cmt, mt, qt, miont);
+        const double r_tp2 = 0.25 * (double)t.ts * (double)t.ts;
         const double eps_self = (double)qt[1];
         if (tid == 0) atomicMax(a.status + 1, max_top);
         if (overflow) {
@@ -1586,19 +1676,18 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
         if (DUMP) {                                              // raw bins, as the sweep reads them
             double* out = a.bins_out + (size_t)q * 3 * nbins;
             for (int b = tid; b < nbins; b += NT) {
-                out[b] = bins_a[b];
-                out[nbins + b] = bins_eps[b];
-                out[2 * nbins + b] = a.use_e ? bins_e[b] : 0.0;
+                out[b] = bins.a[b];
+                out[nbins + b] = bins.eps[b];
+                out[2 * nbins + b] = a.use_e ? bins.e[b] : 0.0;
             }
             if (tid == 0) {
                 a.counts_out[q] = s_nacc;
-                a.eps_self_out[q] = eps_self / ((double)ts * (double)ts);   // reaches the centre as for ts = 1
+                a.eps_self_out[q] = eps_self / ((double)t.ts * (double)t.ts);   // reaches the centre as for ts = 1
                 if (q == 0) { a.scales_out[0] = sc.a; a.scales_out[1] = sc.eps; a.scales_out[2] = sc.e; }
             }
             continue;
         }
-        const double Fk = sweep_rays<MODE, NT>(a, bins_a, bins_eps, bins_e, sc,
-                                                 reinterpret_cast<unsigned char*>(s_node));
+        const double Fk = sweep_rays<MODE, NT>(a, bins.a, bins.eps, bins.e, sc, reinterpret_cast<unsigned char*>(s_nb));
         const double F = block_sum<NT>(Fk, s_red) + eps_self / (4.0 * PI_D * r_tp2);
         if (tid == 0) {
             const int64_t o = a.targets ? q : cell;
@@ -1610,35 +1699,10 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
     if (cur >= 0) flush_counters(a, cnt);
 }
 
-template <int MODE, int OUT, int NT, bool VAR>
-__global__ void __launch_bounds__(NT) k_walk(const WalkArgs* __restrict__ jobs, const int64_t* __restrict__ job_end,
-                                            int n_jobs, unsigned int* counter) {
-    walk_body<MODE, OUT, NT, VAR>(jobs, job_end, n_jobs, counter);
-}
-
-// The double-FP32 form's walk with its CTAs per SM stated: five 128-thread
-// CTAs (its lane-group sweep would otherwise take enough registers to drop
-// it to four), or one wide CTA (left to the default, the compiler aims at two
-// and spills).
-template <int MODE, int OUT, int NT, bool VAR>
-__global__ void __launch_bounds__(NT, NT == 128 ? 5 : 1) k_walk5(const WalkArgs* __restrict__ jobs, const int64_t* __restrict__ job_end,
-                                                 int n_jobs, unsigned int* counter) {
-    walk_body<MODE, OUT, NT, VAR>(jobs, job_end, n_jobs, counter);
-}
-
-template <int MODE, int OUT, int NT, bool VAR>
-constexpr auto walk_kernel() {
-    if constexpr (MODE == 2 && !VAR) return &k_walk5<MODE, OUT, NT, VAR>;
-    else return &k_walk<MODE, OUT, NT, VAR>;
-}
-
-// The same walk with registers capped so that six 128-thread CTAs fit an SM:
-// chosen when the ray bins are small enough for six (N_R <= ~30 at N_PIX 48)
-// and registers would otherwise hold the SM to five.
-template <int MODE, int OUT, int NT, bool VAR>
-__global__ void __launch_bounds__(NT, 6) k_walk_cap6(const WalkArgs* __restrict__ jobs,
-                                                     const int64_t* __restrict__ job_end, int n_jobs,
-                                                     unsigned int* counter) {
+// CTAS: the CTAs per SM that the registers have to allow.
+template <int MODE, int OUT, int NT, int CTAS, bool VAR>
+__global__ void __launch_bounds__(NT, CTAS) k_walk(const WalkArgs* __restrict__ jobs, const int64_t* __restrict__ job_end,
+                                                  int n_jobs, unsigned int* counter) {
     walk_body<MODE, OUT, NT, VAR>(jobs, job_end, n_jobs, counter);
 }
 
@@ -1673,18 +1737,7 @@ __global__ void __launch_bounds__(NT) k_sweep_stored(WalkArgs a, const double* b
     }
 }
 
-constexpr int WALK_NT = 128;                // threads per target (one CTA)
-// Wide CTAs for targets whose ray bins leave room for fewer than three
-// 128-thread CTAs on an SM (N_PIX = 192 with N_R ~ 60 fills most of it):
-// one CTA per SM then brings 16 (FP32 form) or 8 (FP64) warps instead of 4.
-// The FP64 form keeps NT * 12 W_p values in shared memory, hence 256.
-constexpr int WALK_NT_WIDE_F32 = 512;
-constexpr int WALK_NT_WIDE_F64 = 256;
-
-// Opened nodes waiting on a target's stack.  The stack never holds more
-// than the target's opened nodes (a few hundred at theta = 0.5); overflow
-// is detected and reported, never written past.
-constexpr int STACK_CAP = 512;
+constexpr int SWEEP_NT = 128;               // threads per target of the stored-bins sweep
 
 size_t walk_smem(const tr_tree* t) {
     const int nq = t->use_e ? 3 : 2;
@@ -1698,7 +1751,6 @@ WalkArgs make_args(const tr_tree* t) {
     a.kappa = t->kappa;
     a.N = t->N; a.L = t->L; a.nr = t->nr; a.npix = t->npix; a.eta = t->p.eta_r; a.nside = t->p.nside;
     a.use_e = t->use_e;
-    a.stack_cap = STACK_CAP;
     a.th_lim2 = t->p.theta_lim * t->p.theta_lim;
     a.th_if2 = t->p.theta_if * t->p.theta_if;
     a.th_src2 = t->p.theta_src * t->p.theta_src;
@@ -1728,19 +1780,6 @@ WalkArgs make_args(const tr_tree* t) {
 template <int NT, typename K>
 tr_status launch_persistent(K kernel, size_t smem, const WalkArgs* jobs, const int64_t* job_end, int n_jobs,
                             int64_t total, unsigned int* counter, cudaStream_t st) {
-    {
-        int dev = 0, optin = 0;
-        cudaFuncAttributes fa{};
-        cudaGetDevice(&dev);
-        tr_status c = cuda_check(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev),
-                                 "shared memory limit");
-        if (c == TR_OK) c = cuda_check(cudaFuncGetAttributes(&fa, kernel), "kernel attributes");
-        if (c != TR_OK) return c;
-        if (smem + fa.sharedSizeBytes > (size_t)optin)
-            return set_error(TR_EUNSUPPORTED,
-                             "ray bins need %zu + %zu bytes of shared memory per target, more than the %d a CTA can have"
-                             " (fewer rays, a shorter L_ray or no e_prev)", smem, (size_t)fa.sharedSizeBytes, optin);
-    }
     tr_status s = cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                              "cudaFuncSetAttribute(smem)");
     if (s != TR_OK) return s;
@@ -1758,74 +1797,88 @@ tr_status launch_persistent(K kernel, size_t smem, const WalkArgs* jobs, const i
     return cuda_check(cudaGetLastError(), "walk kernel launch");
 }
 
-template <int MODE>
-bool wide_ctas_m(size_t smem) {
+// Warps that one SM holds of a walk kernel with `smem` bytes of bins and
+// buffer (0: it does not fit).
+template <int NT, typename K>
+int resident_warps(K kernel, size_t smem) {
     int per_sm = 0;
-    const void* k = (const void*)walk_kernel<MODE, OUT_FUSED, WALK_NT, false>();
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, WALK_NT, smem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem) != cudaSuccess) {
         cudaGetLastError();
-        return true;                                             // too large for 128 threads: try wide
+        return 0;
     }
-    return per_sm < 3;
+    return per_sm * (NT / 32);
 }
 
-bool wide_ctas(int mode, size_t smem) {
-    return mode == 0 ? wide_ctas_m<0>(smem) : (mode == 1 ? wide_ctas_m<1>(smem) : wide_ctas_m<2>(smem));
+// The walk kernel of one form and output, in the CTA size that puts the most
+// warps on an SM, the smaller one of equals: the walk waits on memory and on
+// its barriers, and the ray bins' shared memory sets how many targets an SM
+// holds.  128 threads: five CTAs at 33 KB of bins (N_PIX 48, N_R 43), six
+// when the bins leave room (N_R <= ~30: 64^3 and 32^3 grids 6% faster than
+// with five); 256 and 512 when the bins fill half or most of an SM (N_PIX
+// 192).  At equal warps the smaller CTA waits less at its barriers
+// (turbulent128: 128 x 5 225 ms, 256 x 4 238 ms).  MODE 2 (double-FP32
+// sweep) only differs from MODE 1 in the sweep, so its dump and
+// column-density walks are those of MODE 1 (chosen by launch_jobs).
+template <int MODE, int OUT, bool VAR>
+tr_status launch_sized(size_t smem, const WalkArgs* jobs, const int64_t* job_end, int n_jobs, int64_t total,
+                       unsigned int* counter, cudaStream_t st) {
+    auto* const k5 = k_walk<MODE, OUT, 128, 5, VAR>;
+    if constexpr (OUT == OUT_CD) return launch_persistent<128>(k5, smem, jobs, job_end, n_jobs, total, counter, st);
+    auto* const k256 = k_walk<MODE, OUT, 256, 2, VAR>;
+    int best = resident_warps<128>(k5, smem), pick = 0;
+    auto better = [&](int w, int k) { if (w > best) { best = w; pick = k; } };
+    if constexpr (OUT == OUT_FUSED && MODE != 0) better(resident_warps<128>(k_walk<MODE, OUT, 128, 6, VAR>, smem), 1);
+    better(resident_warps<256>(k256, smem), 2);
+    if constexpr (MODE != 0) better(resident_warps<512>(k_walk<MODE, OUT, 512, 1, VAR>, smem), 3);
+    if constexpr (OUT == OUT_FUSED && MODE != 0)
+        if (pick == 1) return launch_persistent<128>(k_walk<MODE, OUT, 128, 6, VAR>, smem, jobs, job_end, n_jobs, total, counter, st);
+    if constexpr (MODE != 0)
+        if (pick == 3) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR>, smem, jobs, job_end, n_jobs, total, counter, st);
+    if (pick == 2) return launch_persistent<256>(k256, smem, jobs, job_end, n_jobs, total, counter, st);
+    return launch_persistent<128>(k5, smem, jobs, job_end, n_jobs, total, counter, st);
 }
 
-// whether the register-capped walk fits more CTAs per SM than the plain one
-bool more_ctas_capped(const void* plain, const void* capped, size_t smem) {
-    int a = 0, b = 0;
-    if (cudaFuncSetAttribute(plain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(capped, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, plain, WALK_NT, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, capped, WALK_NT, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return b > a;
-}
-
-// The walk kernel of one form and output.  MODE 2 (double-FP32 sweep) only
-// differs from MODE 1 in the sweep, so its dump and column-density walks are
-// those of MODE 1 (chosen by launch_jobs).
 template <int MODE, bool VAR>
-tr_status launch_mode(int out, bool wide, size_t smem, const WalkArgs* jobs, const int64_t* job_end, int n_jobs,
-                      int64_t total, unsigned int* counter, cudaStream_t st) {
-    constexpr int W = MODE == 0 ? WALK_NT_WIDE_F64 : WALK_NT_WIDE_F32, T = WALK_NT;
-    constexpr int F = OUT_FUSED;
+tr_status launch_mode(int out, size_t smem, const WalkArgs* jobs, const int64_t* job_end, int n_jobs, int64_t total,
+                      unsigned int* counter, cudaStream_t st) {
     if constexpr (MODE != 2) {
-        constexpr int D = OUT_DUMP, C = OUT_CD;
-        if (out == C) return launch_persistent<T>(walk_kernel<MODE, C, T, VAR>(), smem, jobs, job_end, n_jobs, total, counter, st);
-        if (out == D)
-            return wide ? launch_persistent<W>(walk_kernel<MODE, D, W, VAR>(), smem, jobs, job_end, n_jobs, total, counter, st)
-                        : launch_persistent<T>(walk_kernel<MODE, D, T, VAR>(), smem, jobs, job_end, n_jobs, total, counter, st);
+        if (out == OUT_CD) return launch_sized<MODE, OUT_CD, VAR>(smem, jobs, job_end, n_jobs, total, counter, st);
+        if (out == OUT_DUMP) return launch_sized<MODE, OUT_DUMP, VAR>(smem, jobs, job_end, n_jobs, total, counter, st);
     }
-    if (wide) return launch_persistent<W>(walk_kernel<MODE, F, W, VAR>(), smem, jobs, job_end, n_jobs, total, counter, st);
-    if constexpr (MODE != 0) {
-        if (more_ctas_capped((const void*)walk_kernel<MODE, F, T, VAR>(), (const void*)k_walk_cap6<MODE, F, T, VAR>, smem))
-            return launch_persistent<T>(k_walk_cap6<MODE, F, T, VAR>, smem, jobs, job_end, n_jobs, total, counter, st);
-    }
-    return launch_persistent<T>(walk_kernel<MODE, F, T, VAR>(), smem, jobs, job_end, n_jobs, total, counter, st);
+    return launch_sized<MODE, OUT_FUSED, VAR>(smem, jobs, job_end, n_jobs, total, counter, st);
 }
 
 template <bool VAR>
-tr_status launch_jobs_v(int mode, int out, bool wide, size_t smem, const WalkArgs* jobs, const int64_t* job_end,
+tr_status launch_jobs_v(int mode, int out, size_t smem, const WalkArgs* jobs, const int64_t* job_end,
                         int n_jobs, int64_t total, unsigned int* counter, cudaStream_t st) {
-    if (mode == 0) return launch_mode<0, VAR>(out, wide, smem, jobs, job_end, n_jobs, total, counter, st);
+    if (mode == 0) return launch_mode<0, VAR>(out, smem, jobs, job_end, n_jobs, total, counter, st);
     if (mode == 1 || out != OUT_FUSED)
-        return launch_mode<1, VAR>(out, wide, smem, jobs, job_end, n_jobs, total, counter, st);
-    return launch_mode<2, VAR>(out, wide, smem, jobs, job_end, n_jobs, total, counter, st);
+        return launch_mode<1, VAR>(out, smem, jobs, job_end, n_jobs, total, counter, st);
+    return launch_mode<2, VAR>(out, smem, jobs, job_end, n_jobs, total, counter, st);
 }
+
+// Shared memory of a CTA that is not for ray bins and the node buffer: what
+// the 512-thread FP32 and 256-thread FP64 walks take at most, and so the
+// limit on a target's bins whichever CTA size is picked.
+constexpr size_t OWN_SMEM_F32 = 19072, OWN_SMEM_F64 = 40512;
 
 // var: some job uses a kernel choice other than W_p / W_f,3 or a boundary
 // other than isolated
 tr_status launch_jobs(int mode, int out, bool var, size_t smem, const WalkArgs* jobs, const int64_t* job_end,
                       int n_jobs, int64_t total, unsigned int* counter, cudaStream_t st) {
-    const bool wide = out != OUT_CD && wide_ctas(out == OUT_FUSED ? mode : (mode != 0 ? 1 : 0), smem);
-    return var ? launch_jobs_v<true>(mode, out, wide, smem, jobs, job_end, n_jobs, total, counter, st)
-               : launch_jobs_v<false>(mode, out, wide, smem, jobs, job_end, n_jobs, total, counter, st);
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    tr_status c = cuda_check(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev),
+                             "shared memory limit");
+    if (c != TR_OK) return c;
+    const size_t own = out == OUT_CD ? 0 : (mode == 0 ? OWN_SMEM_F64 : OWN_SMEM_F32);
+    if (smem + own > (size_t)optin)
+        return set_error(TR_EUNSUPPORTED,
+                         "ray bins need %zu + %zu bytes of shared memory per target, more than the %d a CTA can have"
+                         " (fewer rays, a shorter L_ray or no e_prev)", smem, own, optin);
+    return var ? launch_jobs_v<true>(mode, out, smem, jobs, job_end, n_jobs, total, counter, st)
+               : launch_jobs_v<false>(mode, out, smem, jobs, job_end, n_jobs, total, counter, st);
 }
 
 bool uses_variants(const tr_tree* t) {
@@ -1927,8 +1980,8 @@ tr_status sweep_run(const tr_rays* r, double* F, double* e, uint8_t* ion, cudaSt
     a.F = F; a.E = e; a.ion = ion;
     a.scales_in = r->scales;
     const size_t smem = (size_t)(r->use_e ? 3 : 2) * r->npix * r->nr * 8 + sweep_scratch_bytes(r->npix);
-    auto kern = r->mode == 0 ? k_sweep_stored<0, WALK_NT>
-                             : (r->mode == 1 ? k_sweep_stored<1, WALK_NT> : k_sweep_stored<2, WALK_NT>);
+    auto kern = r->mode == 0 ? k_sweep_stored<0, SWEEP_NT>
+                             : (r->mode == 1 ? k_sweep_stored<1, SWEEP_NT> : k_sweep_stored<2, SWEEP_NT>);
     tr_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                              "cudaFuncSetAttribute(sweep smem)");
     if (s != TR_OK) return s;
@@ -1936,7 +1989,7 @@ tr_status sweep_run(const tr_rays* r, double* F, double* e, uint8_t* ion, cudaSt
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t blocks = r->n_targets < (int64_t)sms * 4 ? r->n_targets : (int64_t)sms * 4;
-    if (blocks > 0) kern<<<(unsigned)blocks, WALK_NT, smem, st>>>(a, r->bins, r->eps_self);
+    if (blocks > 0) kern<<<(unsigned)blocks, SWEEP_NT, smem, st>>>(a, r->bins, r->eps_self);
     return cuda_check(cudaGetLastError(), "sweep kernel launch");
 }
 
