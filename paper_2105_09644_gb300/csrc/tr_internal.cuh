@@ -88,10 +88,9 @@ struct SweepTables {                        // depend on (N_R, eta_R, N_side, N_
     double* inv_r2 = nullptr;               // 1/r_j^2 (0 for j = 0)
     double* inv_vol = nullptr;              // 1 / ray-cell volume (cells^-3), 4pi/N_PIX shells
     float* inv_volf = nullptr;              // the same in FP32
-    double* G = nullptr;                    // [i][j] (1/2) dV_ij zeta_g,ij (Eq. 14-16)
-    double* ID2 = nullptr;                  // [i][j] 1/(r_j - r_mid,i)^2
-    double* GI = nullptr;                   // [i][j] G_ij ID2_ij
-    float* Gf = nullptr;                    // FP32 copies of G, ID2, GI
+    double* ID2 = nullptr;                  // [i][j] 1/(r_j - r_mid,i)^2, 0 for j <= i
+    double* GI = nullptr;                   // [i][j] G_ij ID2_ij, G_ij = (1/2) dV_ij zeta_g,ij (Eq. 14-16)
+    float* Gf = nullptr;                    // G, ID2, GI in FP32
     float* ID2f = nullptr;
     float* GIf = nullptr;
     double* HT = nullptr;                   // [j][i] (G_{i-1,j} + G_{i,j}) / V_i: lone-source loss per raw deposit

@@ -36,8 +36,7 @@ constexpr size_t OFF_RF = up(OFF_R + sizeof(double) * MAX_NR);
 constexpr size_t OFF_INVR2 = up(OFF_RF + sizeof(float) * MAX_NR);
 constexpr size_t OFF_INVVOL = up(OFF_INVR2 + sizeof(double) * MAX_NR);
 constexpr size_t OFF_INVVOLF = up(OFF_INVVOL + sizeof(double) * MAX_NR);
-constexpr size_t OFF_G = up(OFF_INVVOLF + sizeof(float) * MAX_NR);
-constexpr size_t OFF_ID2 = up(OFF_G + sizeof(double) * NR2);
+constexpr size_t OFF_ID2 = up(OFF_INVVOLF + sizeof(float) * MAX_NR);
 constexpr size_t OFF_GI = up(OFF_ID2 + sizeof(double) * NR2);
 constexpr size_t OFF_GF = up(OFF_GI + sizeof(double) * NR2);
 constexpr size_t OFF_ID2F = up(OFF_GF + sizeof(float) * NR2);
@@ -117,7 +116,6 @@ extern "C" tr_status tr_solve_noalloc(const tr_grid* g, const tr_sources* s, con
         ds.sw.inv_r2 = at<double>(ds.base, OFF_INVR2);
         ds.sw.inv_vol = at<double>(ds.base, OFF_INVVOL);
         ds.sw.inv_volf = at<float>(ds.base, OFF_INVVOLF);
-        ds.sw.G = at<double>(ds.base, OFF_G);
         ds.sw.ID2 = at<double>(ds.base, OFF_ID2);
         ds.sw.GI = at<double>(ds.base, OFF_GI);
         ds.sw.Gf = at<float>(ds.base, OFF_GF);

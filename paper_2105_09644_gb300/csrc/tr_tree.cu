@@ -331,7 +331,7 @@ __device__ __forceinline__ double seg_geom(int i, int j, int nr, int eta, int ns
 }
 
 __global__ void k_sweep_tables(int nr, int eta, int nside, int npix, int zeta_g, double* r, float* rf,
-                               double* inv_r2, double* inv_vol, float* inv_volf, double* G, double* ID2, double* GI,
+                               double* inv_r2, double* inv_vol, float* inv_volf, double* ID2, double* GI,
                                float* Gf, float* ID2f, float* GIf, double* HT) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     auto rad = [eta](int i) { return (double)((int64_t)i * i) / (2.0 * (double)eta * (double)eta); };
@@ -354,7 +354,6 @@ __global__ void k_sweep_tables(int nr, int eta, int nside, int npix, int zeta_g,
             const double rm = 0.5 * (rad(i) + rad(i + 1)), rj = rad(j);
             id2 = 1.0 / ((rj - rm) * (rj - rm));
         }
-        G[t] = g;
         ID2[t] = id2;
         GI[t] = g * id2;
         Gf[t] = (float)g;
@@ -388,7 +387,6 @@ tr_status sweep_tables_make(SweepTables* sw, int nr, int eta, int nside, int npi
         cudaMalloc(&sw->inv_r2, sizeof(double) * nr) != cudaSuccess ||
         cudaMalloc(&sw->inv_vol, sizeof(double) * nr) != cudaSuccess ||
         cudaMalloc(&sw->inv_volf, sizeof(float) * nr) != cudaSuccess ||
-        cudaMalloc(&sw->G, sizeof(double) * n2) != cudaSuccess ||
         cudaMalloc(&sw->ID2, sizeof(double) * n2) != cudaSuccess ||
         cudaMalloc(&sw->GI, sizeof(double) * n2) != cudaSuccess ||
         cudaMalloc(&sw->Gf, sizeof(float) * n2) != cudaSuccess ||
@@ -400,7 +398,7 @@ tr_status sweep_tables_make(SweepTables* sw, int nr, int eta, int nside, int npi
         return set_error(TR_ENOMEM, "cannot allocate the ray tables (N_R = %d)", nr);
     }
     k_sweep_tables<<<grid_for((int64_t)n2, 128), 128, 0, st>>>(nr, eta, nside, npix, zeta_g, sw->r, sw->rf,
-                                                                sw->inv_r2, sw->inv_vol, sw->inv_volf, sw->G, sw->ID2, sw->GI,
+                                                                sw->inv_r2, sw->inv_vol, sw->inv_volf, sw->ID2, sw->GI,
                                                                 sw->Gf, sw->ID2f, sw->GIf, sw->HT);
     s = cuda_check(cudaGetLastError(), "ray table kernel");
     if (s != TR_OK) return s;
@@ -411,8 +409,7 @@ tr_status sweep_tables_make(SweepTables* sw, int nr, int eta, int nside, int npi
 tr_status sweep_tables_fill(SweepTables* sw, int nr, int eta, int nside, int npix, int zeta_g, cudaStream_t st) {
     const size_t n2 = (size_t)nr * nr;
     k_sweep_tables<<<grid_for((int64_t)n2, 128), 128, 0, st>>>(nr, eta, nside, npix, zeta_g, sw->r, sw->rf,
-                                                                sw->inv_r2, sw->inv_vol, sw->inv_volf, sw->G, sw->ID2,
-                                                                sw->GI, sw->Gf, sw->ID2f, sw->GIf, sw->HT);
+                                                                sw->inv_r2, sw->inv_vol, sw->inv_volf, sw->ID2, sw->GI, sw->Gf, sw->ID2f, sw->GIf, sw->HT);
     tr_status s = cuda_check(cudaGetLastError(), "ray table kernel");
     if (s != TR_OK) return s;
     sw->nr = nr; sw->eta = eta; sw->nside = nside; sw->zeta_g = zeta_g;
@@ -421,7 +418,7 @@ tr_status sweep_tables_fill(SweepTables* sw, int nr, int eta, int nside, int npi
 
 void sweep_tables_free(SweepTables* sw) {
     cudaFree(sw->r); cudaFree(sw->rf); cudaFree(sw->inv_r2); cudaFree(sw->inv_vol); cudaFree(sw->inv_volf);
-    cudaFree(sw->G); cudaFree(sw->ID2); cudaFree(sw->GI); cudaFree(sw->Gf); cudaFree(sw->ID2f); cudaFree(sw->GIf);
+    cudaFree(sw->ID2); cudaFree(sw->GI); cudaFree(sw->Gf); cudaFree(sw->ID2f); cudaFree(sw->GIf);
     cudaFree(sw->HT);
     *sw = SweepTables();
 }

@@ -23,9 +23,10 @@
 // for the emission eps), with shared-memory atomics into the ray bins: FP64
 // adds in the FP64 form, exact 64-bit fixed point in the FP32 forms.
 // Sweep (Sec. 2.5, Eq. 12-17): each ray is swept far to near (FP64 and
-// FP32 + FP64-sweep forms: a thread per ray, FP64 arithmetic; FP32 +
-// double-FP32-sweep form: two lanes per ray, FP32 losses, double-FP32
-// budgets) and the CTA sums the rays (Eq. 18).
+// FP32 + FP64-sweep forms: FP64 arithmetic, a lane per ray of few sources
+// and a lane pair per other ray; FP32 + double-FP32-sweep form: FP32 losses,
+// double-FP32 budgets, a lane per source or a pair per ray) and the CTA sums
+// the rays (Eq. 18).
 // Variants: CTAs of 128, 256 or 512 threads by the room that the bins leave,
 // a dump mode keeping the raw bins and accepted ids, a column-density mode
 // without radial points, and a separate instantiation for non-default
@@ -66,13 +67,12 @@ struct WalkArgs {
     const double* inv_r2;
     const double* inv_vol;
     const float* inv_volf;
-    const double* G;
+    const double* HT;                       // [j][i] lone-source loss per raw recombination deposit
     const double* ID2;
     const double* GI;
     const float* Gf;
     const float* ID2f;
     const float* GIf;
-    const double* HT;                       // [j][i] lone-source loss per raw recombination deposit
     const int64_t* targets;                 // NULL: cells first .. first+n_targets-1 in walk order
     int64_t first;
     const uint8_t* flags;                   // AMR tree: node topology (NULL: uniform grid)
@@ -221,11 +221,14 @@ __device__ __forceinline__ float fixed_scale(float total) {
     return ldexpf(1.0f, min(62 - ex, 126));
 }
 
+// A bin times f: FP32 forms, f holds the reciprocal of the unit (a power of two).
 template <int MODE>
-__device__ __forceinline__ double bin_value(const double* slot, float scale) {
-    if (MODE == 0) return *slot;
+__device__ __forceinline__ double bin_value(const double* slot, double f) {
+    if (MODE == 0) return *slot * f;
     const uint2 v = *reinterpret_cast<const uint2*>(slot);
-    return ((double)v.y * 4294967296.0 + (double)v.x) / (double)scale;
+    // 2^84 + high x 2^32 and 2^52 + low, without a conversion
+    const double h = __hiloint2double(0x45300000, (int)v.y), l = __hiloint2double(0x43300000, (int)v.x);
+    return ((h - 19342813118337666422669312.0) + l) * f;
 }
 
 template <int MODE>
@@ -641,27 +644,20 @@ __device__ __forceinline__ int eps_split(const WalkArgs& a, typename Prec<MODE>:
     return i;
 }
 
-// 1/a in FP64 by the Newton-Raphson iteration y <- y + y (1 - a y), seeded with
-// the correctly rounded FP32 reciprocal: the relative error squares at each
-// step (2^-23 -> 2^-46 -> below FP64 rounding), two steps suffice.
-__device__ __forceinline__ double recip_nr(double a) {
-    const float af = (float)a;
-    if (!(fabsf(af) > 1e-30f && fabsf(af) < 1e30f)) return 1.0 / a;
-    double y = (double)__frcp_rn(af);
-    double e = fma(-a, y, 1.0);
-    y = fma(y, e, y);
-    e = fma(-a, y, 1.0);
-    return fma(y, e, y);
+// 1/a in FP64 for a normal a > 0: the hardware's approximation (measured: off
+// by 2^-19.9 at most) and one step of third order, y (1 + e + e^2) with e = 1 -
+// a y (measured: within 2^-52).  Three FP64 instructions.
+__device__ __forceinline__ double recip(double a) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
 
-// The same after one step: relative error about 2^-46, far below the
-// rounding that the inputs of the loss coefficient A zeta_d / F_tot already
-// carry, and two FP64 instructions fewer per segment of the sweep.
-__device__ __forceinline__ double recip1(double a) {
-    const float af = (float)a;
-    if (!(fabsf(af) > 1e-30f && fabsf(af) < 1e30f)) return 1.0 / a;
-    const double y = (double)__frcp_rn(af);
-    return fma(y, fma(-a, y, 1.0), y);
+// A float >= 0 as a double, by integer operations (subnormals give 0).
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f);
+    return b < 0x00800000u ? 0.0 : __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
 // Recombination coefficient per unit volume at point i of a ray.  In the
@@ -671,109 +667,132 @@ __device__ __forceinline__ double recip1(double a) {
 template <int MODE>
 __device__ __forceinline__ double alpha_at(const WalkArgs& a, const double* ba, int i, float inv_scale) {
     if (MODE == 0) return ba[i] * __ldg(a.inv_vol + i);
-    return (double)(bin_value_f<MODE>(ba + i, inv_scale) * __ldg(a.inv_volf + i));
+    return widen(bin_value_f<MODE>(ba + i, inv_scale) * __ldg(a.inv_volf + i));
 }
 
-// Far-to-near sweep of one ray (Sec. 2.5) straight from its bins, by a pair
-// of lanes of one warp (gl = 0, 1; gmask = the pair): ba, be, bee are the
-// ray's N_R slots of alpha, eps and e (raw deposits).  Lane gl owns the
-// ray's source points j with j % 2 == gl and keeps their photon rates Phi_j
-// (FP64, in place of their eps slots); the total flux of a segment (zeta_s,
-// zeta_d) is summed over the pair with one shuffle.  All of it is FP64
-// arithmetic (the FP32 forms' coefficients widened).  The loss of source j
-// over segment i is R_ij = (alpha_i + alpha_{i+1}) G_ij zeta_d zeta_s with
-// G_ij = (1/2) dV_ij zeta_g,ij (Eq. 14-16), and Phi_j <- max(Phi_j - R_ij,
-// 0) (Eq. 13) is one FMA and a test of the sign bit.  GB300 issues FP64 at
-// 1/64 of the FP32 rate and a deep chain of dependent FP64 operations per
-// segment sets the sweep's time, so the pair halves that chain.  Rays
-// without emission cost only the scan for it.  Both lanes return F_0.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
 
+// GB300's FP64: each of an SM's four schedulers has a unit that takes 64 cycles
+// per warp instruction, however many lanes it has, with no overlap (measured:
+// 65 cycles per FMA for one warp, dependent or not; 16 per SM with four warps).
+// So FP64 work is packed onto few warps, those warps lie on different
+// schedulers from one CTA of an SM to the next, and conversions and
+// comparisons go to the integer units.
+
+// Flux at r = 0 of a ray with a lone source at jtop and no e, by a whole warp
+// (lane 0 returns it): zeta_s = zeta_d = 1 on every segment and every R_ij >=
+// 0, so that clipping once at the end equals clipping per segment (Eq. 13):
+// Phi_0 = max(Phi_j - sum_i bin_i HT[j][i], 0).
+template <int MODE>
+__device__ __forceinline__ double lone_ray(const WalkArgs& a, const double* ba, const double* be, const Scales& sc, int jtop) {
+    const int lane = threadIdx.x & 31;
+    const float ia = 1.0f / sc.a;
+    const double* h = a.HT + (size_t)jtop * a.nr;
+    double s0 = 0.0;
+    for (int i = lane; i <= jtop; i += 32)
+        s0 = fma(MODE == 0 ? ba[i] : widen(bin_value_f<MODE>(ba + i, ia)), __ldg(h + i), s0);
+    s0 = warp_sum(s0);
+    const double phi = bin_value<MODE>(be + jtop, (MODE == 0 ? 1.0 : 1.0 / (double)sc.eps) * (1.0 / (4.0 * PI_D))) - s0;
+    return positive(phi) && lane == 0 ? phi * __ldg(a.inv_r2 + jtop) : 0.0;
+}
+
+// Readies one ray for the FP64 sweep, by a whole warp (a lane per segment, so
+// that the FP64 units see one instruction for 32 segments): leaves in ba[i],
+// i < jtop, the loss coefficient A_i = alpha_i + alpha_{i+1} of segment i (Eq.
+// 14; G carries the 1/2).  With the energy density e, zeta_d = min(2, F_tot /
+// e) (Eq. 17), so the loss per unit of F_j G_ij is A zeta_d / F_tot = min(2 A /
+// F_tot, A / e): where e > 0 at the segment's far point, ba[i] holds 2 A and
+// bee[i] the limit A / e (else infinity).
+template <int MODE>
+__device__ __forceinline__ void prepare_ray(const WalkArgs& a, double* ba, double* bee, const Scales& sc, int jtop) {
+    const int lane = threadIdx.x & 31;
+    const float ia = 1.0f / sc.a, ie = 1.0f / sc.e;
+    for (int base = 0; base < jtop; base += 32) {
+        const int i = base + lane;
+        double A = 0.0, Q = 0.0;
+        if (i < jtop) {
+            A = alpha_at<MODE>(a, ba, i, ia) + alpha_at<MODE>(a, ba, i + 1, ia);
+            if (bee) {
+                const double ev = alpha_at<MODE>(a, bee, i + 1, ie);
+                Q = __longlong_as_double(0x7ff0000000000000LL);
+                if (positive(ev)) { Q = A * recip(ev); A = A + A; }
+            }
+        }
+        __syncwarp();                                         // raw values read before they are replaced
+        if (i < jtop) { ba[i] = A; if (bee) bee[i] = Q; }
+        __syncwarp();
+    }
+}
+
+__device__ __forceinline__ int farthest(uint64_t m0, uint64_t m1) {
+    return m1 ? 127 - __clzll((long long)m1) : (m0 ? 63 - __clzll((long long)m0) : 0);
+}
+
+// min(cf, limit): both >= 0, so their bit patterns compare like them.
+__device__ __forceinline__ double loss_coef(double cf, const double* bee, int i) {
+    if (!bee) return cf;
+    const long long x = __double_as_longlong(cf), y = __double_as_longlong(bee[i]);
+    return __longlong_as_double(x < y ? x : y);
+}
+
+// FP64 sweep of one ray with any number of emitting points (m0, m1) by a pair
+// of lanes of one warp (gl = 0, 1; gmask = the pair).  ba holds the ray's raw
+// alpha deposits, or after prepare_ray (`ready`; always with e) its loss
+// coefficients, bee then the limits on the loss; be its raw eps deposits.
+// Lane gl owns the ray's source points j with j %
+// 2 == gl and keeps their photon rates Phi_j (FP64, in place of their eps
+// slots); the total flux of a segment (zeta_s, zeta_d) is summed over the
+// pair with one shuffle.  The loss of source j over segment i is R_ij =
+// (alpha_i + alpha_{i+1}) G_ij zeta_d zeta_s with G_ij = (1/2) dV_ij
+// zeta_g,ij (Eq. 14-16), and Phi_j <- max(Phi_j - R_ij, 0) (Eq. 13) is one
+// FMA and a test of the sign bit.  Bound by the FP64 units: three
+// instructions per source and segment.  Both lanes return F_0.
 constexpr uint64_t EVEN_BITS = 0x5555555555555555ull;   // bits j with j % 2 == 0
 
 template <int MODE>
-__device__ __forceinline__ double sweep_ray(const WalkArgs& a, const double* ba, double* be, const double* bee, const Scales& sc,
-                            int gl, unsigned gmask) {
+__device__ __forceinline__ double sweep_ray(const WalkArgs& a, const double* ba, double* be, const double* bee,
+                                            const Scales& sc, uint64_t m0, uint64_t m1, int gl, unsigned gmask, bool ready) {
     const int nr = a.nr;
-    uint64_t m0 = 0, m1 = 0;
-    for (int j = 2 - gl; j < nr; j += 2) {                    // lane gl scans its parity (j >= 1)
-        if (bin_nonzero<MODE>(be + j)) { if (j < 64) m0 |= 1ull << j; else m1 |= 1ull << (j - 64); }
-    }
-    m0 |= __shfl_xor_sync(gmask, m0, 1);
-    m1 |= __shfl_xor_sync(gmask, m1, 1);
-    if (!(m0 | m1)) return 0.0;
     const uint64_t sel = EVEN_BITS << gl;                     // the lane's parity (64 is even)
     uint64_t o0 = m0 & sel, o1 = m1 & sel;                    // own live sources
-    const double inv4pi = 1.0 / (4.0 * PI_D);
-    for (uint64_t w = o0; w; w &= w - 1) { const int j = __ffsll((long long)w) - 1; be[j] = bin_value<MODE>(be + j, sc.eps) * inv4pi; }
-    for (uint64_t w = o1; w; w &= w - 1) { const int j = 64 + __ffsll((long long)w) - 1; be[j] = bin_value<MODE>(be + j, sc.eps) * inv4pi; }
+    const double f4pi = (MODE == 0 ? 1.0 : 1.0 / (double)sc.eps) * (1.0 / (4.0 * PI_D));
+    for (uint64_t w = o0; w; w &= w - 1) { const int j = __ffsll((long long)w) - 1; be[j] = bin_value<MODE>(be + j, f4pi); }
+    for (uint64_t w = o1; w; w &= w - 1) { const int j = 64 + __ffsll((long long)w) - 1; be[j] = bin_value<MODE>(be + j, f4pi); }
     double* ph = be;                                              // Eq. 12
-    __syncwarp(gmask);
-    const float ia = 1.0f / sc.a, ie = 1.0f / sc.e;
-    const int jtop = m1 ? 64 + 63 - __clzll((long long)m1) : 63 - __clzll((long long)m0);
-    if (!bee && __popcll((long long)m0) + __popcll((long long)m1) == 1) {
-        // a lone source and no e: zeta_s = zeta_d = 1 on every segment, every
-        // R_ij >= 0, so clipping once at the end equals clipping per segment
-        // (Eq. 13): Phi_0 = max(Phi_j - sum_i bin_i HT[j][i], 0), an FP64 dot
-        // product split over the pair
-        const double* h = a.HT + (size_t)jtop * nr;
-        double s0 = 0.0;
-        for (int i = gl; i <= jtop; i += 2)
-            s0 = fma((double)(MODE == 0 ? ba[i] : (double)bin_value_f<MODE>(ba + i, ia)), __ldg(h + i), s0);
-        s0 += __shfl_xor_sync(gmask, s0, 1);
-        const double phi = ph[jtop] - s0;
-        return positive(phi) ? phi * __ldg(a.inv_r2 + jtop) : 0.0;
-    }
-    double a_hi = alpha_at<MODE>(a, ba, jtop, ia);
+    const int jtop = farthest(m0, m1);
+    const float ia = 1.0f / sc.a;
+    double a_hi = ready ? 0.0 : alpha_at<MODE>(a, ba, jtop, ia);
     for (int i = jtop - 1; i >= 0; --i) {
+        double A = ba[i];
+        if (!ready) {                                             // (in the shadow of the FP64 chain)
+            const double a_lo = alpha_at<MODE>(a, ba, i, ia);
+            A = a_lo + a_hi;
+            a_hi = a_lo;
+        }
         const int b = i + 1;                                      // sources strictly beyond r_i
         const uint64_t a0 = (b < 64) ? (o0 & (~0ull << b)) : 0ull;
         const uint64_t a1 = (b <= 64) ? o1 : (o1 & (~0ull << (b - 64)));
-        const int own = __popcll((long long)a0) + __popcll((long long)a1);
-        const int cnt = own + __shfl_xor_sync(gmask, own, 1);
-        if (cnt == 0) {                                           // nothing left beyond r_i on the ray
-            if (!__any_sync(gmask, (o0 | o1) != 0ull)) break;
-            a_hi = alpha_at<MODE>(a, ba, i, ia);
-            continue;
-        }
-        const double a_lo = alpha_at<MODE>(a, ba, i, ia);
-        const double A = a_lo + a_hi;                             // twice the mean coefficient
-        if (!bee && cnt == 1) {
-            // one source on the segment: zeta_s = 1, and zeta_d = 1 without e
-            if (own) {
-                const int j = a0 ? __ffsll((long long)a0) - 1 : 64 + __ffsll((long long)a1) - 1;
-                const double np = fma(-A, __ldg(a.G + (size_t)i * nr + j), ph[j]);   // Eq. 13-14
-                if (positive(np)) ph[j] = np;
-                else { ph[j] = 0.0; if (j < 64) o0 &= ~(1ull << j); else o1 &= ~(1ull << (j - 64)); }
+        const double* id2 = a.ID2 + (size_t)i * nr;
+        const double* gi = a.GI + (size_t)i * nr;
+        double Fl = 0.0;                                          // Eq. 11 at the segment midpoint
+        for (uint64_t w = a0; w; w &= w - 1) { const int j = __ffsll((long long)w) - 1; Fl = fma(ph[j], __ldg(id2 + j), Fl); }
+        for (uint64_t w = a1; w; w &= w - 1) { const int j = 64 + __ffsll((long long)w) - 1; Fl = fma(ph[j], __ldg(id2 + j), Fl); }
+        const double Ftot = Fl + __shfl_xor_sync(gmask, Fl, 1);
+        if (positive(Ftot)) {
+            const double cf = loss_coef(A * recip(Ftot), bee, i);   // zeta_s = F_j / Ftot (Eq. 16)
+            for (uint64_t w = a0; w; w &= w - 1) {
+                const int j = __ffsll((long long)w) - 1;
+                const double np = fma(-cf * __ldg(gi + j), ph[j], ph[j]);   // Eq. 13-14
+                if (positive(np)) ph[j] = np; else { ph[j] = 0.0; o0 &= ~(1ull << j); }
             }
-        } else {
-            const double* id2 = a.ID2 + (size_t)i * nr;
-            const double* gi = a.GI + (size_t)i * nr;
-            double Fl = 0.0;                                      // Eq. 11 at the segment midpoint
-            for (uint64_t w = a0; w; w &= w - 1) { const int j = __ffsll((long long)w) - 1; Fl = fma(ph[j], __ldg(id2 + j), Fl); }
-            for (uint64_t w = a1; w; w &= w - 1) { const int j = 64 + __ffsll((long long)w) - 1; Fl = fma(ph[j], __ldg(id2 + j), Fl); }
-            const double Ftot = Fl + __shfl_xor_sync(gmask, Fl, 1);
-            if (positive(Ftot)) {
-                const double inv_F = recip1(Ftot);
-                double zd = 1.0;                                  // Eq. 17
-                if (bee) {
-                    const double ev = alpha_at<MODE>(a, bee, i + 1, ie);
-                    if (positive(ev)) zd = fmin(2.0, Ftot * recip_nr(ev));
-                }
-                const double cf = bee ? A * zd * inv_F : A * inv_F;   // zeta_s = F_j / Ftot (Eq. 16)
-                for (uint64_t w = a0; w; w &= w - 1) {
-                    const int j = __ffsll((long long)w) - 1;
-                    const double np = fma(-cf * __ldg(gi + j), ph[j], ph[j]);   // Eq. 13-14
-                    if (positive(np)) ph[j] = np; else { ph[j] = 0.0; o0 &= ~(1ull << j); }
-                }
-                for (uint64_t w = a1; w; w &= w - 1) {
-                    const int j = 64 + __ffsll((long long)w) - 1;
-                    const double np = fma(-cf * __ldg(gi + j), ph[j], ph[j]);
-                    if (positive(np)) ph[j] = np; else { ph[j] = 0.0; o1 &= ~(1ull << (j - 64)); }
-                }
+            for (uint64_t w = a1; w; w &= w - 1) {
+                const int j = 64 + __ffsll((long long)w) - 1;
+                const double np = fma(-cf * __ldg(gi + j), ph[j], ph[j]);
+                if (positive(np)) ph[j] = np; else { ph[j] = 0.0; o1 &= ~(1ull << (j - 64)); }
             }
+        } else if (!__any_sync(gmask, (o0 | o1) != 0ull)) {
+            break;                                                // nothing left beyond or before r_i on the ray
         }
-        a_hi = a_lo;
     }
     double F0 = 0.0;                                              // Eq. 10-11 at r = 0
     for (uint64_t w = o0; w; w &= w - 1) { const int j = __ffsll((long long)w) - 1; F0 = fma(ph[j], __ldg(a.inv_r2 + j), F0); }
@@ -812,26 +831,18 @@ constexpr int SG = 2;
 constexpr uint64_t SG_PATTERN = 0x5555555555555555ull;   // bits j with j % 2 == 0
 
 __device__ __forceinline__ double sweep_ray_group(const WalkArgs& a, const double* ba, double* be, const double* bee,
-                                  const Scales& sc, int gl, unsigned gmask) {
+                                  const Scales& sc, uint64_t m0, uint64_t m1, int gl, unsigned gmask) {
     const int nr = a.nr;
-    uint64_t m0 = 0, m1 = 0;
-    for (int j = 1 + ((gl + SG - 1) % SG); j < nr; j += SG) {   // lane gl scans j == gl (mod SG)
-        if (bin_nonzero<1>(be + j)) { if (j < 64) m0 |= 1ull << j; else m1 |= 1ull << (j - 64); }
-    }
-    for (int o = 1; o < SG; o <<= 1) {
-        m0 |= __shfl_xor_sync(gmask, m0, o);
-        m1 |= __shfl_xor_sync(gmask, m1, o);
-    }
     if (!(m0 | m1)) return 0.0;
     const uint64_t sel = SG_PATTERN << gl;                    // 64 % SG == 0: same pattern for m1
     const uint64_t o0 = m0 & sel, o1 = m1 & sel;
-    const double inv4pi = 1.0 / (4.0 * PI_D);
+    const double inv_eps = 1.0 / (double)sc.eps, inv4pi = 1.0 / (4.0 * PI_D);
     float2* E = reinterpret_cast<float2*>(be);
     float2* Ls = reinterpret_cast<float2*>(const_cast<double*>(ba));
     for (int half = 0; half < 2; ++half)
         for (uint64_t w = half ? o1 : o0; w; w &= w - 1) {
             const int j = (half ? 64 : 0) + __ffsll((long long)w) - 1;
-            const double v = bin_value<1>(be + j, sc.eps) * inv4pi;   // Eq. 12
+            const double v = bin_value<1>(be + j, inv_eps) * inv4pi;   // Eq. 12
             const float hi = (float)v;
             E[j] = make_float2(hi, (float)(v - (double)hi));
         }
@@ -908,61 +919,192 @@ __device__ __forceinline__ double sweep_ray_group(const WalkArgs& a, const doubl
     return F0;
 }
 
-// Per-target ray tables for the double-FP32 sweep, in shared scratch:
-// order[npix] (u16, the ray of each rank), off[npix] (u16, first lane of each
-// lane group), cnt[npix] (u8, emitting points of each ray), then four ints:
-// the rays with sources, the lanes of the groups, the rays swept by pairs,
-// the emitting points of all rays.
+// Per-target ray tables for the sweep, in shared scratch: cls (per chunk of 16
+// rays and class, the rays of that class, one bit per two lanes), npts (per
+// chunk, emitting points), order (u16, the ray of each rank), off (u16, first
+// lane of each lane group), m1 (emitting points 64 and beyond, with N_R > 64
+// only).
 constexpr int MAX_NPIX = 12 * 8 * 8;                  // N_side <= 8
 constexpr int GROUP_MAX = 32;                         // rays with more points go to lane pairs
 constexpr int GROUP_MEAN_MAX = 14;                    // lane groups while a lit ray has at most this many points on average
-__host__ __device__ constexpr size_t sweep_hdr_offset(int npix) { return ((size_t)npix * 5 + 3) & ~(size_t)3; }
-__host__ __device__ constexpr size_t sweep_scratch_bytes(int npix) { return sweep_hdr_offset(npix) + 16; }
+constexpr int N_CLS = 7;                              // classes of rays with emitting points
+struct RayScratch {
+    uint32_t* cls;
+    int* npts;
+    uint64_t* m1;
+    uint16_t *order, *off;
+};
+__host__ __device__ constexpr size_t ray_chunks(int npix) { return ((size_t)npix + 15) / 16; }
+__host__ __device__ constexpr size_t sweep_scratch_bytes(int npix, int nr) {
+    return (nr > 64 ? (size_t)npix * 8 : 0) + ray_chunks(npix) * (N_CLS + 1) * 4 + (size_t)npix * 4;
+}
+__device__ __forceinline__ RayScratch ray_scratch(unsigned char* p, int npix, int nr) {
+    RayScratch rs;
+    rs.m1 = reinterpret_cast<uint64_t*>(p);
+    rs.cls = reinterpret_cast<uint32_t*>(p + (nr > 64 ? (size_t)npix * 8 : 0));
+    rs.npts = reinterpret_cast<int*>(rs.cls + ray_chunks(npix) * N_CLS);
+    rs.order = reinterpret_cast<uint16_t*>(rs.npts + ray_chunks(npix));
+    rs.off = rs.order + npix;
+    return rs;
+}
+
+// The emitting points of ray k, as ray_census left them: points below 64 in
+// the ray's eps slot 0 (a deposit there is at the target itself and not swept).
+__device__ __forceinline__ void ray_mask(const double* bins_eps, const RayScratch& rs, int nr, int k, uint64_t& m0,
+                                         uint64_t& m1) {
+    m0 = *reinterpret_cast<const uint64_t*>(bins_eps + (size_t)k * nr);
+    m1 = nr > 64 ? rs.m1[k] : 0ull;
+}
 
 // Lanes given to a ray with c emitting points in a lane group: the next
 // power of two.
 __device__ __forceinline__ int group_width(int c) { return c <= 1 ? c : 1 << (32 - __clz(c - 1)); }
 
-// Ranks the rays of a target for the double-FP32 sweep, ties by ray index:
-// first the rays with more than GROUP_MAX emitting points (swept by lane
-// pairs), then the others by decreasing lane-group width, each group's first
-// lane recorded (groups sorted by decreasing power-of-two width never
-// straddle a warp), rays without sources last.  Deterministic: the ranks
-// depend only on the bins.
-template <int NT>
-__device__ __forceinline__ void rank_rays(const WalkArgs& a, const double* bins_eps, unsigned char* scratch) {
-    const int npix = a.npix, nr = a.nr, tid = threadIdx.x;
-    uint16_t* order = reinterpret_cast<uint16_t*>(scratch);
-    uint16_t* off = order + npix;
-    uint8_t* cnt = reinterpret_cast<uint8_t*>(off + npix);
-    int* hdr = reinterpret_cast<int*>(scratch + sweep_hdr_offset(npix));
-    for (int k = tid; k < npix; k += NT) {
-        const double* be = bins_eps + (size_t)k * nr;
-        int c = 0;
-        for (int j = 1; j < nr; ++j) c += bin_nonzero<1>(be + j) ? 1 : 0;
-        cnt[k] = (uint8_t)c;
-    }
-    __syncthreads();                                          // counts visible
-    auto key = [](int c) { return c > GROUP_MAX ? 2 * GROUP_MAX : group_width(c); };
-    for (int k = tid; k < npix; k += NT) {
-        const int ck = key(cnt[k]);
-        int rank = 0, lanes = 0, nz = 0, total = 0, nbig = 0, npts = 0;
-        for (int k2 = 0; k2 < npix; ++k2) {
-            const int c2 = cnt[k2], key2 = key(c2);
-            const bool before = key2 > ck || (key2 == ck && k2 < k);
-            const int w2 = c2 > GROUP_MAX ? 0 : key2;
-            rank += before ? 1 : 0;
-            lanes += before ? w2 : 0;
-            total += w2;
-            nz += c2 > 0 ? 1 : 0;
-            nbig += c2 > GROUP_MAX ? 1 : 0;
-            npts += c2;
+// Class of a ray by its emitting points c: 0 more than GROUP_MAX, then by
+// decreasing group width 32, 16, .. 1; -1: no points.
+__device__ __forceinline__ int ray_class(int c) {
+    if (c == 0) return -1;
+    return c > GROUP_MAX ? 0 : 1 + __clz(c == 1 ? 1 : 2 * c - 1) - 26;
+}
+
+struct Ranks { int nz, lanes, nbig, none, npts; };    // rays with points, lanes of the groups, rays of more than
+                                                      // GROUP_MAX points and of one point, points of all rays
+
+// Finds each ray's emitting points (a lane pair per ray) and ranks the rays
+// by class, ties by ray index: deterministic, so that sums over the rays are.
+// The lane groups, sorted by decreasing power-of-two width, never straddle a
+// warp.  Two barriers, no loop over the other rays
+// (counting by one thread per ray and comparing all pairs of rays took 3 k
+// warp instructions per target at N_PIX 48).
+template <int MODE, int NT>
+__device__ __forceinline__ Ranks rank_rays(const WalkArgs& a, double* bins_eps, const RayScratch& rs) {
+    const int npix = a.npix, nr = a.nr, tid = threadIdx.x, lane = tid & 31, gl = tid & 1;
+    for (int k = tid >> 1; k < (int)ray_chunks(npix) * 16; k += NT / 2) {   // warp-uniform: 16 rays
+        uint64_t m0 = 0, m1 = 0;
+        double* be = bins_eps + (size_t)k * nr;
+        if (k < npix)
+            for (int j = 2 - gl; j < nr; j += 2)               // lane gl scans its parity (j >= 1)
+                if (bin_nonzero<MODE>(be + j)) { if (j < 64) m0 |= 1ull << j; else m1 |= 1ull << (j - 64); }
+        m0 |= __shfl_xor_sync(FULL, m0, 1);
+        m1 |= __shfl_xor_sync(FULL, m1, 1);
+        const int c = __popcll((long long)m0) + __popcll((long long)m1);
+        const int cls = ray_class(c), chunk = k >> 4;
+        const int sum = __reduce_add_sync(FULL, gl ? 0 : c);
+        if (k < npix && gl == 0) {
+            *reinterpret_cast<uint64_t*>(be) = m0;
+            if (nr > 64) rs.m1[k] = m1;
         }
-        order[rank] = (uint16_t)k;
-        off[rank] = (uint16_t)lanes;
-        if (k == 0) { hdr[0] = nz; hdr[1] = total; hdr[2] = nbig; hdr[3] = npts; }
+        for (int q = 0; q < N_CLS; ++q) {
+            const unsigned m = __ballot_sync(FULL, cls == q && gl == 0);
+            if (lane == 0) rs.cls[chunk * N_CLS + q] = m;
+        }
+        if (lane == 0) rs.npts[chunk] = sum;
+    }
+    __syncthreads();                                          // masks and class bits visible
+    const int nch = (int)ray_chunks(npix);
+    Ranks r{0, 0, 0, 0, 0};
+    for (int ch = 0; ch < nch; ++ch) {
+        r.npts += rs.npts[ch];
+        for (int q = 0; q < N_CLS; ++q) {
+            const int n = __popc(rs.cls[ch * N_CLS + q]);
+            r.nz += n;
+            if (q == 0) r.nbig += n;
+            else r.lanes += n << (6 - q);
+            if (q == N_CLS - 1) r.none += n;
+        }
+    }
+    for (int k = tid; k < npix; k += NT) {
+        uint64_t m0, m1;
+        ray_mask(bins_eps, rs, nr, k, m0, m1);
+        const int cls = ray_class(__popcll((long long)m0) + __popcll((long long)m1));
+        if (cls < 0) continue;
+        int rank = 0, lanes = 0;
+        for (int ch = 0; ch < nch; ++ch)
+            for (int q = 0; q <= cls; ++q) {
+                unsigned m = rs.cls[ch * N_CLS + q];
+                if (q == cls && ch >= (k >> 4)) m = ch > (k >> 4) ? 0u : m & ((1u << (2 * (k & 15))) - 1u);
+                const int n = __popc(m);
+                rank += n;
+                if (q > 0) lanes += n << (6 - q);
+            }
+        rs.order[rank] = (uint16_t)k;
+        rs.off[rank] = (uint16_t)lanes;
     }
     __syncthreads();                                          // ranks visible
+    return r;
+}
+
+// The lane group that group-lane p of T belongs to: its ray k, the ray's points
+// c, the group's width w, the lane's place in it, its own point jA (0: none)
+// and the ray's farthest.  Returns whether p < T.
+__device__ __forceinline__ bool group_lane(const double* bins_eps, const RayScratch& rs, const Ranks& rk, int nr, int p, int T,
+                                           int& k, int& c, int& w, int& slot, int& jA, int& jtop) {
+    const bool in = p < T;
+    int g = rk.nbig;                                          // the last rank whose group starts at or before p
+    uint64_t m0 = 0, m1 = 0;
+    k = slot = 0;
+    if (in) {
+        int hi = rk.nz - 1;
+        while (g < hi) {
+            const int mid = (g + hi + 1) >> 1;
+            if ((int)rs.off[mid] <= p) g = mid; else hi = mid - 1;
+        }
+        k = rs.order[g];
+        slot = p - (int)rs.off[g];
+        ray_mask(bins_eps, rs, nr, k, m0, m1);
+    }
+    c = __popcll((long long)m0) + __popcll((long long)m1);
+    w = group_width(c);
+    jtop = farthest(m0, m1);
+    for (int n = 0; n < slot; ++n) { if (m0) m0 &= m0 - 1; else m1 &= m1 - 1; }
+    jA = m0 ? __ffsll((long long)m0) - 1 : (m1 ? 63 + __ffsll((long long)m1) : 0);
+    return in;
+}
+
+// FP64 sweep, after prepare_ray, of 32 group lanes from `base` on: a lane per
+// emitting point of the rays with up to GROUP_MAX points, its Phi_j in a
+// register, the segments far to near in lockstep over the warp.  A segment's
+// total flux is a butterfly sum over the group.  The tables hold zero for
+// points not beyond the segment and a spent source is zero, so nothing is
+// masked.  6 + log2(w) FP64 instructions per segment for 32 points; the tables
+// are loaded a segment ahead.  Each group's first lane returns its ray's F_0.
+template <int MODE>
+__device__ __forceinline__ double sweep_group64(const WalkArgs& a, const double* bins_a, const double* bins_eps,
+                                                const double* bins_e, const Scales& sc, const RayScratch& rs,
+                                                const Ranks& rk, int base, int T) {
+    const int nr = a.nr, lane = threadIdx.x & 31;
+    int k, c, w, slot, jA, jtop;
+    const bool in = group_lane(bins_eps, rs, rk, nr, base + lane, T, k, c, w, slot, jA, jtop);
+    const double* ba = bins_a + (size_t)k * nr;
+    const double* bee = bins_e ? bins_e + (size_t)k * nr : nullptr;
+    double ph = 0.0;
+    if (jA > 0) ph = bin_value<MODE>(bins_eps + (size_t)k * nr + jA, (MODE == 0 ? 1.0 : 1.0 / (double)sc.eps) * (1.0 / (4.0 * PI_D)));
+    const int wmax = __reduce_max_sync(FULL, (unsigned)w);
+    const int itop = __reduce_max_sync(FULL, (unsigned)jtop);
+    const double* id2p = a.ID2 + (size_t)(itop - 1) * nr + jA;
+    const double* gip = a.GI + (size_t)(itop - 1) * nr + jA;
+    double id2 = __ldg(id2p), gi = __ldg(gip);
+    for (int i = itop - 1; i >= 0; --i) {
+        const double id2c = id2, gic = gi;
+        if (i > 0) { id2p -= nr; gip -= nr; id2 = __ldg(id2p); gi = __ldg(gip); }
+        double F = ph * id2c;                                 // Eq. 11 at the segment midpoint
+        for (int o = 1; o < wmax; o <<= 1) {
+            const double t = __shfl_xor_sync(FULL, F, o);
+            if (o < w) F += t;
+        }
+        if (positive(F)) {
+            const double cf = loss_coef(ba[i] * recip(F), bee, i);   // zeta_s = F_j / F_tot (Eq. 16)
+            const double np = fma(-cf * gic, ph, ph);         // Eq. 13-14
+            ph = positive(np) ? np : 0.0;
+        }
+        if (!__any_sync(FULL, positive(ph))) break;           // every point of the warp spent
+    }
+    double F0 = ph * __ldg(a.inv_r2 + jA);                    // Eq. 10-11 at r = 0
+    for (int o = 1; o < wmax; o <<= 1) {
+        const double t = __shfl_xor_sync(FULL, F0, o);
+        if (o < w) F0 += t;
+    }
+    return in && slot == 0 ? F0 : 0.0;
 }
 
 // Double-FP32 sweep of the rays of a target with 1..GROUP_MAX emitting
@@ -979,47 +1121,20 @@ __device__ __forceinline__ void rank_rays(const WalkArgs& a, const double* bins_
 // Each group's first lane returns its ray's F_0 (FP64) in the sum.
 template <int NT>
 __device__ __forceinline__ double sweep_groups(const WalkArgs& a, const double* bins_a, const double* bins_eps, const double* bins_e,
-                               const Scales& sc, const unsigned char* scratch) {
-    const int npix = a.npix, nr = a.nr, lane = threadIdx.x & 31;
-    const uint16_t* order = reinterpret_cast<const uint16_t*>(scratch);
-    const uint16_t* off = order + npix;
-    const uint8_t* cnt = reinterpret_cast<const uint8_t*>(off + npix);
-    const int* hdr = reinterpret_cast<const int*>(scratch + sweep_hdr_offset(npix));
-    const int nz = hdr[0], T = hdr[1], nbig = hdr[2];
-    const double inv4pi = 1.0 / (4.0 * PI_D);
+                               const Scales& sc, const RayScratch& rs, const Ranks& rk) {
+    const int nr = a.nr, lane = threadIdx.x & 31, T = rk.lanes;
+    const double inv_eps = 1.0 / (double)sc.eps, inv4pi = 1.0 / (4.0 * PI_D);
     const float ia = 1.0f / sc.a, ie = 1.0f / sc.e;
     double Fk = 0.0;
     for (int base = threadIdx.x & ~31; base < T; base += NT) {  // warp-uniform
-        const int p = base + lane;
-        const bool in = p < T;
-        int g = nbig;                                         // the last rank whose group starts at or before p
-        if (in) {
-            int hi = nz - 1;
-            while (g < hi) {
-                const int mid = (g + hi + 1) >> 1;
-                if ((int)off[mid] <= p) g = mid; else hi = mid - 1;
-            }
-        }
-        const int k = in ? order[g] : 0;
-        const int c = in ? cnt[k] : 0;
-        const int w = group_width(c);
-        const int slot = in ? p - (int)off[g] : 0;
+        int k, c, w, slot, jA, jtop;
+        const bool in = group_lane(bins_eps, rs, rk, nr, base + lane, T, k, c, w, slot, jA, jtop);
         const double* ba = bins_a + (size_t)k * nr;
         const double* be = bins_eps + (size_t)k * nr;
         const double* bee = bins_e ? bins_e + (size_t)k * nr : nullptr;
-        int jA = 0, jtop = 0;                                 // own point, the ray's farthest
-        if (in) {
-            int n = 0;
-            for (int j = 1; j < nr; ++j)
-                if (bin_nonzero<1>(be + j)) {
-                    if (n == slot) jA = j;
-                    jtop = j;
-                    ++n;
-                }
-        }
         const bool vA = slot < c;
         float2 EA = make_float2(0.f, 0.f), LA = EA;
-        if (vA) { const double v = bin_value<1>(be + jA, sc.eps) * inv4pi; EA.x = (float)v; EA.y = (float)(v - (double)EA.x); }
+        if (vA) { const double v = bin_value<1>(be + jA, inv_eps) * inv4pi; EA.x = (float)v; EA.y = (float)(v - (double)EA.x); }
         bool sA = !vA;                                        // spent, or no point
         const bool single = c == 1 && !bee;                   // zeta_s = zeta_d = 1 throughout
         const int wmax = __reduce_max_sync(FULL, (unsigned)w);
@@ -1068,64 +1183,92 @@ __device__ __forceinline__ double sweep_groups(const WalkArgs& a, const double* 
     return Fk;
 }
 
-// Sum over the rays of one target (Eq. 18).  FP64 sweeps (FP64 form and
-// FP32 + FP64-sweep form): a pair of consecutive lanes per ray -- GB300
-// charges an FP64 warp instruction in full however few lanes it has, so the
-// FP64 work is packed onto consecutive lanes.  Double-FP32 sweep, ranked by
-// rank_rays: a target whose lit rays carry more than GROUP_MEAN_MAX emitting
-// points on average is swept by lane pairs (sweep_ray_group); otherwise its
-// rays with more than GROUP_MAX points by lane pairs and the others a lane per
-// point (sweep_groups).  The choice depends only on the bins.  `scratch` holds
-// sweep_scratch_bytes(npix) bytes of shared memory; all threads call.
+// Sum over the rays of one target (Eq. 18), ranked by rank_rays; `turn`
+// rotates which warps take the work from target to target.
+// FP64 sweeps (FP64 form and FP32 + FP64-sweep form): rays with a lone source
+// by a warp each (lone_ray).  Of the others, while their points fill at most
+// one lane group position per thread of the CTA, all warps ready the rays
+// (prepare_ray) and sweep them a lane per point (sweep_group64; more than
+// GROUP_MAX points: lane pairs): the fewest FP64 instructions in a row, and the
+// target's time is that chain.  Beyond that the FP64 units are what is short,
+// and lane pairs, 16 rays of like load to a warp, take fewest in all (a lane
+// for a point that the sweep has not reached costs as much as a busy one).
+// turbulent128 278 -> 236 ms with this rule, 275 with pairs only, 251 with half
+// the threads as the line; AMR 64^3 at N_PIX 192 35 ms with groups only, 24
+// with the rule.  Coefficients computed within the chain where lane pairs
+// sweep: 505 -> 492 ms for 10^4 sources at 128^3 (its FP64 units are busy).
+// Double-FP32 sweep: lane groups up to GROUP_MEAN_MAX points per lit ray on
+// average (sweep_groups), lane pairs beyond (sweep_ray_group).  The choices
+// depend only on the bins.  `scratch` holds sweep_scratch_bytes bytes of
+// shared memory; all threads call.
 template <int MODE, int NT>
 __device__ __forceinline__ double sweep_rays(const WalkArgs& a, double* bins_a, double* bins_eps, double* bins_e,
-                                             const Scales& sc, unsigned char* scratch) {
+                                             const Scales& sc, unsigned char* scratch, int turn) {
     const int nr = a.nr, tid = threadIdx.x, lane = tid & 31;
+    constexpr int NW = NT / 32;
+    const RayScratch rs = ray_scratch(scratch, a.npix, nr);
+    const bool use_e = a.use_e != 0;
+    const Ranks rk = rank_rays<MODE, NT>(a, bins_eps, rs);
     double Fk = 0.0;
+    uint64_t m0 = 0, m1 = 0;
     if constexpr (MODE != 2) {
+        const int wid = ((tid >> 5) + turn) & (NW - 1);       // its place in the sum too (block_sum)
+        const int n_lone = use_e ? 0 : rk.none, T = rk.lanes - n_lone, n_more = rk.nz - n_lone;
+        const bool groups = T <= NT, ready = groups || use_e;
+        for (int r = (ready ? 0 : n_more) + wid; r < rk.nz; r += NW) {
+            const int k = rs.order[r];
+            ray_mask(bins_eps, rs, nr, k, m0, m1);
+            const int jtop = farthest(m0, m1);
+            if (r < n_more) prepare_ray<MODE>(a, bins_a + k * nr, use_e ? bins_e + k * nr : nullptr, sc, jtop);
+            else Fk += lone_ray<MODE>(a, bins_a + k * nr, bins_eps + k * nr, sc, jtop);
+        }
+        if (ready) __syncthreads();                           // coefficients visible
+        const int n_pair = groups ? rk.nbig : n_more;
         const int gl = tid & 1;
         const unsigned gmask = 3u << (lane & ~1);
-        for (int k = tid >> 1; k < a.npix; k += NT / 2) {
-            const double f = sweep_ray<MODE>(a, bins_a + k * nr, bins_eps + k * nr, a.use_e ? bins_e + k * nr : nullptr,
-                                             sc, gl, gmask);
+        for (int r = wid * 16 + (lane >> 1); r < n_pair; r += NT / 2) {
+            const int k = rs.order[r];
+            ray_mask(bins_eps, rs, nr, k, m0, m1);
+            const double f = sweep_ray<MODE>(a, bins_a + k * nr, bins_eps + k * nr, use_e ? bins_e + k * nr : nullptr,
+                                             sc, m0, m1, gl, gmask, ready);
             if (gl == 0) Fk += f;
         }
+        if (groups)
+            for (int base = (NW - 1 - wid) * 32; base < T; base += NT)
+                Fk += sweep_group64<MODE>(a, bins_a, bins_eps, use_e ? bins_e : nullptr, sc, rs, rk, base, T);
         return Fk;
     } else {
-    rank_rays<NT>(a, bins_eps, scratch);
-    const uint16_t* order = reinterpret_cast<const uint16_t*>(scratch);
-    const int* hdr = reinterpret_cast<const int*>(scratch + sweep_hdr_offset(a.npix));
     const int gl = tid % SG;
     const unsigned gmask = ((1u << SG) - 1u) << (lane & ~(SG - 1));
-    if (hdr[3] > GROUP_MEAN_MAX * hdr[0]) {
+    if (rk.npts > GROUP_MEAN_MAX * rk.nz) {
         // many points per ray: every ray by lane pairs, in ray order (ranked
         // order would put the heaviest rays in one warp, which then holds
         // the CTA's barrier)
         for (int k = tid / SG; k < a.npix; k += NT / SG) {
-            const double f = sweep_ray_group(a, bins_a + k * nr, bins_eps + k * nr,
-                                             a.use_e ? bins_e + k * nr : nullptr, sc, gl, gmask);
+            ray_mask(bins_eps, rs, nr, k, m0, m1);
+            const double f = sweep_ray_group(a, bins_a + k * nr, bins_eps + k * nr, use_e ? bins_e + k * nr : nullptr,
+                                             sc, m0, m1, gl, gmask);
             if (gl == 0) Fk += f;
         }
         return Fk;
     }
     // the pair-swept rays round-robin over the warps, so that no warp holds
     // the CTA's barrier with all of them
-    constexpr int NW = NT / 32;
-    const int nbig = hdr[2];
-    for (int r = (tid >> 5) + NW * (lane / SG); r < nbig; r += NT / SG) {
-        const int k = order[r];
-        const double f = sweep_ray_group(a, bins_a + k * nr, bins_eps + k * nr,
-                                         a.use_e ? bins_e + k * nr : nullptr, sc, gl, gmask);
+    for (int r = (tid >> 5) + NW * (lane / SG); r < rk.nbig; r += NT / SG) {
+        const int k = rs.order[r];
+        ray_mask(bins_eps, rs, nr, k, m0, m1);
+        const double f = sweep_ray_group(a, bins_a + k * nr, bins_eps + k * nr, use_e ? bins_e + k * nr : nullptr,
+                                         sc, m0, m1, gl, gmask);
         if (gl == 0) Fk += f;
     }
-    return Fk + sweep_groups<NT>(a, bins_a, bins_eps, a.use_e ? bins_e : nullptr, sc, scratch);
+    return Fk + sweep_groups<NT>(a, bins_a, bins_eps, use_e ? bins_e : nullptr, sc, rs, rk);
     }
 }
 
 template <int NT>
-__device__ __forceinline__ double block_sum(double v, double* red) {
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+__device__ __forceinline__ double block_sum(double v, double* red, int turn) {
+    v = warp_sum(v);                                               // (the sum's order follows the rotated warps)
+    const int lane = threadIdx.x & 31, wid = ((threadIdx.x >> 5) + turn) & (NT / 32 - 1);
     if (lane == 0) red[wid] = v;
     __syncthreads();
     double t = 0.0;
@@ -1444,7 +1587,6 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
     __shared__ int s_nacc;
     __shared__ __align__(16) WalkArgs s_a;                       // the current job
     __shared__ NodeBatch<MODE> s_nb[NW];
-    static_assert(sizeof(NodeBatch<MODE>) * NW >= sweep_scratch_bytes(MAX_NPIX), "sweep scratch in s_nb");
     __shared__ uint32_t s_acc[acc_cap<NT>()];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const WalkArgs& a = s_a;
@@ -1687,8 +1829,11 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
             }
             continue;
         }
-        const double Fk = sweep_rays<MODE, NT>(a, bins.a, bins.eps, bins.e, sc, reinterpret_cast<unsigned char*>(s_nb));
-        const double F = block_sum<NT>(Fk, s_red) + eps_self / (4.0 * PI_D * r_tp2);
+        const int turn = MODE == 2 ? 0 : (int)q;
+        static_assert(sizeof s_nb >= sweep_scratch_bytes(MAX_NPIX, 64) && sizeof s_nb >= sweep_scratch_bytes(192, MAX_NR),
+                      "the sweep's tables fit the spread's memory");
+        const double Fk = sweep_rays<MODE, NT>(a, bins.a, bins.eps, bins.e, sc, reinterpret_cast<unsigned char*>(s_nb), turn);
+        const double F = block_sum<NT>(Fk, s_red, turn) + eps_self / (4.0 * PI_D * r_tp2);
         if (tid == 0) {
             const int64_t o = a.targets ? q : cell;
             if (a.F) a.F[o] = F * a.Fconv;
@@ -1725,10 +1870,11 @@ __global__ void __launch_bounds__(NT) k_sweep_stored(WalkArgs a, const double* b
             if (a.use_e) bins_e[b] = in[2 * nbins + b];
         }
         __syncthreads();
+        const int turn = MODE == 2 ? 0 : (int)q;
         const double Fk = sweep_rays<MODE, NT>(a, bins_a, bins_eps, bins_e,
                                                Scales{a.scales_in[0], a.scales_in[1], a.scales_in[2]},
-                                               smem + (size_t)(a.use_e ? 3 : 2) * nbins * sizeof(double));
-        const double F = block_sum<NT>(Fk, s_red) + eps_self[q] / (4.0 * PI_D * 0.25);
+                                               smem + (size_t)(a.use_e ? 3 : 2) * nbins * sizeof(double), turn);
+        const double F = block_sum<NT>(Fk, s_red, turn) + eps_self[q] / (4.0 * PI_D * 0.25);
         if (tid == 0) {
             if (a.F) a.F[q] = F * a.Fconv;
             if (a.E) a.E[q] = F * a.Econv;
@@ -1761,7 +1907,7 @@ WalkArgs make_args(const tr_tree* t) {
     a.lrayf = (float)t->lray;
     a.toff = t->table->off; a.tent = t->table->ent; a.hdr = t->table->hdr;
     a.r = t->sw.r; a.rf = t->sw.rf; a.inv_r2 = t->sw.inv_r2; a.inv_vol = t->sw.inv_vol; a.inv_volf = t->sw.inv_volf;
-    a.G = t->sw.G; a.ID2 = t->sw.ID2; a.GI = t->sw.GI; a.Gf = t->sw.Gf; a.ID2f = t->sw.ID2f; a.GIf = t->sw.GIf;
+    a.ID2 = t->sw.ID2; a.GI = t->sw.GI; a.Gf = t->sw.Gf; a.ID2f = t->sw.ID2f; a.GIf = t->sw.GIf;
     a.HT = t->sw.HT;
     a.Fconv = t->U / (t->dx * t->dx);
     a.Econv = t->Eu;
@@ -1972,14 +2118,14 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
 tr_status sweep_run(const tr_rays* r, double* F, double* e, uint8_t* ion, cudaStream_t st) {
     WalkArgs a{};
     a.nr = r->nr; a.npix = r->npix; a.use_e = r->use_e;
-    a.r = r->sw.r; a.inv_r2 = r->sw.inv_r2; a.inv_vol = r->sw.inv_vol; a.inv_volf = r->sw.inv_volf; a.G = r->sw.G; a.ID2 = r->sw.ID2; a.GI = r->sw.GI; a.Gf = r->sw.Gf; a.ID2f = r->sw.ID2f; a.GIf = r->sw.GIf;
+    a.r = r->sw.r; a.inv_r2 = r->sw.inv_r2; a.inv_vol = r->sw.inv_vol; a.inv_volf = r->sw.inv_volf; a.ID2 = r->sw.ID2; a.GI = r->sw.GI; a.Gf = r->sw.Gf; a.ID2f = r->sw.ID2f; a.GIf = r->sw.GIf;
     a.HT = r->sw.HT;
     a.n_targets = r->n_targets;
     a.Fconv = r->U / (r->dx * r->dx);
     a.Econv = r->Eu;
     a.F = F; a.E = e; a.ion = ion;
     a.scales_in = r->scales;
-    const size_t smem = (size_t)(r->use_e ? 3 : 2) * r->npix * r->nr * 8 + sweep_scratch_bytes(r->npix);
+    const size_t smem = (size_t)(r->use_e ? 3 : 2) * r->npix * r->nr * 8 + sweep_scratch_bytes(r->npix, r->nr);
     auto kern = r->mode == 0 ? k_sweep_stored<0, SWEEP_NT>
                              : (r->mode == 1 ? k_sweep_stored<1, SWEEP_NT> : k_sweep_stored<2, SWEEP_NT>);
     tr_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),

@@ -73,7 +73,7 @@ def footprint_bytes(N: int, precision: int, n_sources: int = 1000, eta_r: int = 
     rounds large allocations to 2 MiB and packs small ones together): the
     library's tree (node records and build sums; the FP32 forms keep the
     FP64 tree beside the FP32 one, and a word for its error bound), mapped
-    emission, status words and counters, the job record, the twelve ray
+    emission, status words and counters, the job record, the eleven ray
     tables; and the request's inputs and outputs.  The node->ray table of
     each N_side is shared by all requests and is not counted here."""
     def rounded(b):
@@ -84,7 +84,7 @@ def footprint_bytes(N: int, precision: int, n_sources: int = 1000, eta_r: int = 
     lib = [n_nodes * 64, n_nodes * 24] if precision == 0 else [n_nodes * 32, n_nodes * 12, n_nodes * 64,
                                                                 n_nodes * 24, 4]
     lib += [cells * 8, 16, 64, 4, 512]                                     # emission, status, stats, counter, job
-    lib += [nr * 8] * 5 + [nr * nr * 8] * 7                                # ray tables
+    lib += [nr * 8] * 5 + [nr * nr * 8] * 6                                # ray tables
     io = [cells * 8, n_sources * 32, cells * 8, cells * 8, cells]          # n_H, sources, F, e, ion
     return sum(rounded(b) for b in lib + io)
 
