@@ -57,7 +57,7 @@ struct Table {                              // CSR: entries of key k are ent[off
 };
 
 __host__ __device__ inline int64_t level_offset(int l) {
-    return ((int64_t(1) << (3 * l)) - 1) / 7;
+    return (int64_t)(0x09249249u & ((1u << (3 * l)) - 1u));     // (8^l - 1) / 7 = 1 + 8 + .. + 8^(l-1), l <= 10
 }
 
 __host__ __device__ inline uint32_t spread3(uint32_t v) {   // 10 bits -> every third bit

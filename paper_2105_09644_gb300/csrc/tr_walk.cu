@@ -105,6 +105,38 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// GB300's FP64: each of an SM's four schedulers has a unit that takes 64 cycles
+// per warp instruction, however many lanes it has, with no overlap (measured:
+// 65 cycles per FMA for one warp, dependent or not; 16 per SM with four warps).
+// So FP64 work is packed onto few warps, those warps lie on different
+// schedulers from one CTA of an SM to the next, and conversions and
+// comparisons go to the integer units.
+
+// 1/a in FP64 for a normal a > 0: the hardware's approximation (measured: off
+// by 2^-19.9 at most) and one step of third order, y (1 + e + e^2) with e = 1 -
+// a y (measured: within 2^-52).  Three FP64 instructions.
+__device__ __forceinline__ double recip(double a) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// A float >= 0 as a double, by integer operations (subnormals give 0).
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f);
+    return b < 0x00800000u ? 0.0 : __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
+// The nearest float towards zero of a double in the float range (bounds only).
+__device__ __forceinline__ float narrow(double a) {
+    return __uint_as_float(((uint32_t)__double2hiint(a) - 0x38000000u) << 3 | (uint32_t)__double2loint(a) >> 29);
+}
+
+// Comparisons of non-negative doubles: their bit patterns order like them.
+__device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool less(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+
 // W_p of App. A (Eq. A2), outer branch rebuilt from the constraints printed
 // with it: W_p2(x) = (x - sqrt3/2)^2 (a2 x + 2A(2 + sqrt3) - a2/2).
 template <typename T>
@@ -122,6 +154,18 @@ __device__ __forceinline__ T wp_kernel(T x) {
         const T outer = t * t * (a2 * x + c2);
         return x < T(0.5) ? inner : (x < s3h ? outer : T(0));
     }
+}
+
+// W_p in FP64 for lanes on either side of its branches: both as k0 + u^2 (k1 +
+// k2 u), u = x or x - sqrt3/2, the constants picked by integer selects.  Four
+// FP64 instructions instead of seven and two comparisons.
+__device__ __forceinline__ double wp_select(double x) {
+    constexpr double a1 = 1.21, a2 = -6.35, A = 4.08, M = 1.184, s3h = 0.86602540378443864676;
+    constexpr double c1 = 0.5 * a1 + 4.0 * (M - A), c2 = 2.0 * A * (2.0 + 1.73205080756887729353) - 0.5 * a2;
+    const bool in = less(x, 0.5);
+    const double u = x - (in ? 0.0 : s3h);
+    const double w = fma(u * u, fma(in ? a1 : a2, u, in ? -c1 : c2 + a2 * s3h), in ? M : 0.0);
+    return less(x, s3h) ? w : 0.0;
 }
 
 // W_g of App. A (Eq. A1): exp(-x^2), truncated at sqrt3/2.
@@ -286,14 +330,15 @@ __device__ __forceinline__ void load_node(const void* nodes, int64_t id, typenam
     }
 }
 
-// Opening decision of a non-leaf node that does not contain the target.
+// Opening decision of a non-leaf node that does not contain the target (an
+// infinite angle always accepts, so its products are not formed).
 __device__ __forceinline__ bool must_open(double h2, double d2, double m, double mion, double eps,
                                           const WalkArgs& a) {
-    const bool acc_lim = h2 < __dmul_rn(a.th_lim2, d2);
-    const bool is_if = (__dmul_rn(DELTA_IF, m) < mion) && (mion < __dmul_rn(1.0 - DELTA_IF, m));
-    const bool acc_if = !is_if || (h2 < __dmul_rn(a.th_if2, d2));
-    const bool acc_src = !(eps > 0.0) || (h2 < __dmul_rn(a.th_src2, d2));
-    return !(acc_lim && acc_if && acc_src);
+    if (!less(h2, __dmul_rn(a.th_lim2, d2))) return true;
+    if (isfinite(a.th_if2f) && __dmul_rn(DELTA_IF, m) < mion && mion < __dmul_rn(1.0 - DELTA_IF, m) &&
+        !less(h2, __dmul_rn(a.th_if2, d2)))
+        return true;
+    return isfinite(a.th_src2f) && positive(eps) && !less(h2, __dmul_rn(a.th_src2, d2));
 }
 // The same decision taken in FP64 with the node's IF flag given (FP32 forms,
 // when FP32 cannot settle it).
@@ -398,9 +443,9 @@ __device__ __forceinline__ T radius_at(int i, T coef, const double* tab) {
 // its edge (the normalisation then jumps between one point and the linear
 // split) -- is not settled in FP32; radial_setup_exact then takes it in FP64.
 template <int MODE>
-__device__ __forceinline__ bool radial_setup(const WalkArgs& a, RadialSpread<MODE>& n, typename Prec<MODE>::real d,
-                                             int s, typename Prec<MODE>::real* wcol, int gauss, float dtol) {
-    using real = typename Prec<MODE>::real;
+__device__ __forceinline__ bool radial_setup(const WalkArgs& a, RadialSpread<MODE>& n, float d, int s, float* wcol, int gauss,
+                                             float dtol) {
+    using real = float;
     const int nr = a.nr;
     const real rc = (MODE == 0) ? (real)a.r_coef : (real)a.r_coeff;
     n.b = real(1); n.lng = false;
@@ -478,10 +523,59 @@ __device__ __forceinline__ int bracket_d(const double* r, int nr, int eta, doubl
     return i;
 }
 
+// The same in FP64, settled always.  Bound by the FP64 units, so six FP64
+// instructions per point (the kernel's argument is one add, r_i / h being exact
+// in FP32; four for the kernel, one for the sum) and none for the index bounds,
+// comparisons and conversions: plain FP64 turbulent64 92 -> 70 ms, Stroemgren
+// 32^3 7.5 -> 5.6 ms.
+__device__ __forceinline__ void radial_setup64(const WalkArgs& a, RadialSpread<0>& n, double d, int s, double* wcol,
+                                               int gauss) {
+    const int nr = a.nr;
+    n.b = 1.0; n.lng = false;
+    if (!less(d, __ldg(a.r + nr - 1))) {
+        n.lo = nr - 1; n.npts = 1; wcol[0] = 1.0;
+        return;
+    }
+    // s is a power of two: 1 / h from its exponent
+    const float hf = (float)s, inv_hf = __uint_as_float((254u << 23) - __float_as_uint(hf));
+    const double h = widen(hf), inv_h = widen(inv_hf), hpar = gauss ? h : inv_h;
+    const float df = narrow(d), reach = 0.8661f * hf, dlo = df > reach ? df - reach : 0.f;
+    const float el = 2.f * dlo, eh = 2.f * (df + reach);
+    const int lo = max((int)((float)a.eta * (el * rsqrtf(fmaxf(el, 1e-30f))) - 1e-3f), 0);
+    const int hi = min((int)((float)a.eta * (eh * rsqrtf(eh)) + 1.001f), nr - 1);
+    double S = 0.0;
+    int cnt = 0, last = lo - 1;
+    double* col = wcol;
+    float fi = (float)lo;
+    const double dh = d * inv_h;            // (exact)
+    const float rch = a.r_coeff * inv_hf;
+    for (int i = lo; i <= hi; ++i, fi += 1.f) {
+        const double w = gauss ? radial_w<double>(fabs(__ldg(a.r + i) - d), hpar, 1)
+                               : wp_select(fabs(widen(fi * fi * rch) - dh));
+        if (positive(w)) {                  // the support is one run of points
+            S += w;
+            last = i;
+            if (cnt < MAXW<0>) *col = w;
+            col += 32;
+            ++cnt;
+        }
+    }
+    if (cnt > 0) {
+        n.lo = last - cnt + 1; n.npts = cnt; n.b = recip(S);
+        if (cnt > MAXW<0>) { n.lng = true; wcol[0] = d; wcol[32] = hpar; }
+        return;
+    }
+    const int i = bracket_d(a.r, nr, a.eta, d);
+    const double ra = __ldg(a.r + i), rb = __ldg(a.r + i + 1);
+    n.lo = i; n.npts = 2;
+    wcol[0] = (rb - d) / (rb - ra);
+    wcol[32] = (d - ra) / (rb - ra);
+}
+
 // FP32 forms: the radial set-up of an accepted node taken on its FP64
 // distance d, when radial_setup could not settle it.  Only the supports
 // that FP32 left open reach here (at most two points, both at the edge, or
-// none), so the weights are stored explicitly: one point (weight 1), two
+// consecutive points, or the linear split between the points bracketing d.
 // consecutive points, or the linear split between the points bracketing d.
 template <int MODE>
 __device__ void radial_setup_exact(const WalkArgs& a, RadialSpread<MODE>& n, double d, int s,
@@ -644,22 +738,6 @@ __device__ __forceinline__ int eps_split(const WalkArgs& a, typename Prec<MODE>:
     return i;
 }
 
-// 1/a in FP64 for a normal a > 0: the hardware's approximation (measured: off
-// by 2^-19.9 at most) and one step of third order, y (1 + e + e^2) with e = 1 -
-// a y (measured: within 2^-52).  Three FP64 instructions.
-__device__ __forceinline__ double recip(double a) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double e = fma(-a, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
-// A float >= 0 as a double, by integer operations (subnormals give 0).
-__device__ __forceinline__ double widen(float f) {
-    const uint32_t b = __float_as_uint(f);
-    return b < 0x00800000u ? 0.0 : __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
-}
-
 // Recombination coefficient per unit volume at point i of a ray.  In the
 // FP32 + FP64-sweep form the deposits are FP32, so the coefficient is formed
 // in FP32 and widened; the photon budget (Phi_j, its losses and their
@@ -669,15 +747,6 @@ __device__ __forceinline__ double alpha_at(const WalkArgs& a, const double* ba, 
     if (MODE == 0) return ba[i] * __ldg(a.inv_vol + i);
     return widen(bin_value_f<MODE>(ba + i, inv_scale) * __ldg(a.inv_volf + i));
 }
-
-__device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
-
-// GB300's FP64: each of an SM's four schedulers has a unit that takes 64 cycles
-// per warp instruction, however many lanes it has, with no overlap (measured:
-// 65 cycles per FMA for one warp, dependent or not; 16 per SM with four warps).
-// So FP64 work is packed onto few warps, those warps lie on different
-// schedulers from one CTA of an SM to the next, and conversions and
-// comparisons go to the integer units.
 
 // Flux at r = 0 of a ray with a lone source at jtop and no e, by a whole warp
 // (lane 0 returns it): zeta_s = zeta_d = 1 on every segment and every R_ij >=
@@ -1415,7 +1484,7 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
             };
             bool in_reach;
             if constexpr (MODE == 0) {
-                in_reach = d <= a.lray;
+                in_reach = !less(a.lray, d);
             } else {
                 if ((float)d + dtol < a.lrayf * (1.f - 2.f * U32)) in_reach = true;
                 else if ((float)d - dtol > a.lrayf * (1.f + 2.f * U32)) in_reach = false;
@@ -1425,7 +1494,7 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
                 const uint2 hd = __ldg(a.hdr + table_key(v.ox, v.oy, v.oz, s));
                 off = hd.x; ne = (int)hd.y;
                 cnt.ent += ne;
-                if (qv[1] != real(0)) {
+                if (MODE == 0 ? positive(qv[1]) : qv[1] != real(0)) {
                     if (VAR && a.kern_e != TR_EPS_WF3) {
                         const double dvar = MODE != 0 ? exact_d() : (double)d;
                         deposit_eps_variant<MODE>(a, bins.eps, off, ne, dvar, qv[1], sc.eps, s);
@@ -1436,9 +1505,10 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
                 }
                 if (qv[0] != real(0) || (a.use_e && qv[2] != real(0))) {
                     const int gauss = VAR ? a.kern_a : 0;
-                    if (radial_setup<MODE>(a, n, d, s, &nb.w[0][lane], gauss, dtol)) {
-                        if constexpr (MODE != 0) radial_setup_exact<MODE>(a, n, exact_d(), s, &nb.w[0][lane], gauss);
-                    }
+                    real* const wcol = &nb.w[0][lane];
+                    if constexpr (MODE == 0) radial_setup64(a, n, d, s, wcol, gauss);
+                    else if (radial_setup<MODE>(a, n, d, s, wcol, gauss, dtol))
+                        radial_setup_exact<MODE>(a, n, exact_d(), s, wcol, gauss);
                     alpha = qv[0];
                     e = a.use_e ? qv[2] : real(0);
                 }
@@ -1501,15 +1571,15 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
         const int b0 = ray * nr + (int)(pk & 0x7fu);
         const real* wc = &nb.w[0][src];
         if constexpr (MODE == 0) {
-            const double c = (double)(ec & 0xffffu);
+            const double c = widen((float)(ec & 0xffffu));
             const double ca = c * nb.a[kc], ce = use_e ? c * nb.e[kc] : 0.0;
             const double d = wc[0], hpar = wc[32];
             for (int j = 0; j < npts; ++j) {
                 const double w = (pk & PK_LONG)
                                      ? radial_w<double>(fabs(radius_at<double>((int)(pk & 0x7fu) + j, a.r_coef, a.r) - d), hpar, VAR ? a.kern_a : 0)
                                      : wc[j * 32];
-                if (ca != 0.0) atomicAdd(bins.a + b0 + j, w * ca);
-                if (use_e && ce != 0.0) atomicAdd(bins.e + b0 + j, w * ce);
+                if (positive(ca)) atomicAdd(bins.a + b0 + j, w * ca);
+                if (use_e && positive(ce)) atomicAdd(bins.e + b0 + j, w * ce);
             }
         } else {
             // ((W b) cnt) (alpha scale / TW): the scales are powers of two
@@ -1686,9 +1756,21 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
         __syncthreads();
         // spread the last `take` listed nodes, 32 per warp at a time
         auto spread_list = [&](int take, int img) {
-            for (int b = nl - take + wid * 32; b < nl; b += NT) {
-                const bool have = b + lane < nl;
-                spread_nodes<MODE, OUT, VAR>(a, s_nb[wid], have ? s_acc[b + lane] : 0u, have, img, t, bins, sc, kap, cnt);
+            if constexpr (CD) {
+                // every node deposits on few rays and siblings on the same ones:
+                // a batch of nodes from all over the list retries fewer FP64
+                // atomics (64^3: 20.7 -> 16.4 ms)
+                const int batches = (take + 31) >> 5;
+                for (int b = wid; b < batches; b += NW) {
+                    const int k = nl - take + b + lane * batches;
+                    const bool have = k < nl;
+                    spread_nodes<MODE, OUT, VAR>(a, s_nb[wid], have ? s_acc[k] : 0u, have, img, t, bins, sc, kap, cnt);
+                }
+            } else {
+                for (int b = nl - take + wid * 32; b < nl; b += NT) {
+                    const bool have = b + lane < nl;
+                    spread_nodes<MODE, OUT, VAR>(a, s_nb[wid], have ? s_acc[b + lane] : 0u, have, img, t, bins, sc, kap, cnt);
+                }
             }
             nl -= take;
         };
