@@ -80,6 +80,19 @@ __host__ __device__ inline uint32_t morton3(uint32_t x, uint32_t y, uint32_t z) 
     return spread3(x) | (spread3(y) << 1) | (spread3(z) << 2);
 }
 
+#ifdef __CUDACC__
+// A float >= 0 as a double, by integer operations (subnormals give 0): GB300's
+// FP64 units also do the conversions, at 64 cycles per warp instruction.
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f);
+    return b < 0x00800000u ? 0.0 : __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+__device__ __forceinline__ double widen_signed(float f) {
+    const double d = widen(fabsf(f));
+    return __hiloint2double(__double2hiint(d) | (int)(__float_as_uint(f) & 0x80000000u), __double2loint(d));
+}
+#endif
+
 // ---- host-side handles ---------------------------------------------------
 struct SweepTables {                        // depend on (N_R, eta_R, N_side, N_PIX, zeta_g)
     int nr = 0, eta = 0, nside = 0, zeta_g = -1;

@@ -38,6 +38,12 @@ __global__ void k_map_sources(double* ndot, int N, double lo0, double lo1, doubl
     atomicAdd(&ndot[(ic[2] * N + ic[1]) * N + ic[0]], Q[s]);
 }
 
+// Level of node `id` in the level-order numbering: (8^l - 1) / 7 <= id, so 7 id
+// + 1 has between 3 l and 3 l + 2 bits below its top bit.
+__device__ __forceinline__ int node_level(int64_t id) {
+    return (63 - __clzll(7 * id + 1)) / 3;
+}
+
 struct F32Sum {                              // Kahan-Neumaier accumulator
     float s = 0.f, c = 0.f;
     __device__ void add(float x) {
@@ -49,46 +55,183 @@ struct F32Sum {                              // Kahan-Neumaier accumulator
     __device__ float value() const { return s + c; }
 };
 
-// Leaves (cells): netting of Eq. 1-2 per cell, e of Eq. 3, ionised mass.
-template <int MODE>
-__global__ void k_leaves(void* nodes_v, void* sums_v, int N, int L, const double* n_H,
-                         const double* ndot, const double* e_prev, double invU, double invEu) {
-    const int64_t nleaf = (int64_t)N * N * N;
-    int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (m >= nleaf) return;
-    const uint32_t ix = compact3((uint32_t)m), iy = compact3((uint32_t)m >> 1), iz = compact3((uint32_t)m >> 2);
-    const int64_t c = ((int64_t)iz * N + iy) * N + ix;
-    const int64_t id = level_offset(L) + m;
-    const double n = n_H[c];
-    const double rec = n * n;                       // alpha_B n^2 dV in units of U
-    const double src = ndot[c] * invU;
-    const double ep = e_prev ? e_prev[c] : 0.0;
-    if (MODE == 0) {
-        NodeF64 nd;
-        nd.m = n;
-        double sx = __dmul_rn(n, (double)ix + 0.5), sy = __dmul_rn(n, (double)iy + 0.5),
-               sz = __dmul_rn(n, (double)iz + 0.5);
-        if (n > 0.0) { nd.cmx = __ddiv_rn(sx, n); nd.cmy = __ddiv_rn(sy, n); nd.cmz = __ddiv_rn(sz, n); }
-        else { nd.cmx = (double)ix + 0.5; nd.cmy = (double)iy + 0.5; nd.cmz = (double)iz + 0.5; }
-        nd.alpha = fmax(rec - src, 0.0);
-        nd.eps = fmax(src - rec, 0.0);
-        nd.e = ep * invEu;
-        nd.mion = (ep > 0.0) ? n : 0.0;
-        ((NodeF64*)nodes_v)[id] = nd;
-        double* sm = (double*)sums_v + 3 * id;
-        sm[0] = sx; sm[1] = sy; sm[2] = sz;
-    } else {
-        NodeF32 nd;                                 // a cell's mass sits at its centre: offset 0
-        const float nf = (float)n;
-        nd.m = nf;
-        nd.ox = 0.f; nd.oy = 0.f; nd.oz = 0.f;
-        nd.alpha = (float)fmax(rec - src, 0.0);
-        nd.eps = (float)fmax(src - rec, 0.0);
-        nd.e = (float)(ep * invEu);
-        nd.mion = (ep > 0.0) ? nf : 0.f;
-        ((NodeF32*)nodes_v)[id] = nd;
-        float* sm = (float*)sums_v + 3 * id;
-        sm[0] = 0.f; sm[1] = 0.f; sm[2] = 0.f;
+// ---- uniform grids: the tree three levels at a time ------------------------
+
+struct BuildArgs {
+    NodeF64* n64;                           // the FP64 tree (the whole tree, or the sidecar of the FP32 forms)
+    double* s64;                            // first moments of the nodes that the next launch starts from
+    NodeF32* n32;
+    float* s32;
+    float* kappa;
+    const double* n_H;
+    const double* ndot;
+    const double* e_prev;
+    double invU, invEu;
+    int N, lc;                              // level of the launch's children
+};
+
+constexpr int BUILD_NT = 512;               // children of a CTA: an 8^3 block of them
+// fields of a node in shared memory, padded so that the eight children of
+// consecutive parents lie in different banks
+enum { B_M, B_X, B_Y, B_Z, B_ALPHA, B_EPS, B_E, B_MION, B_FIELDS };
+constexpr int BUILD_PAD = BUILD_NT + BUILD_NT / 8;
+__device__ __forceinline__ int padded(int i) { return i + (i >> 3); }
+
+// Centre of mass m p / m of a cell at p (a half integer): p itself unless the
+// rounding of the product moves the quotient to a neighbour, which its exact
+// residual r decides: |r| / m below half an ulp of p.  Two FP64 instructions
+// instead of a division.
+__device__ __forceinline__ double cell_centre(double m, float pf, double& mp) {
+    const double p = widen(pf);
+    mp = __dmul_rn(m, p);
+    if (!(__double2hiint(m) > 0x10000000)) return m > 0.0 ? __ddiv_rn(mp, m) : p;   // tiny or no mass
+    const double r = fabs(fma(-m, p, mp));
+    const int e = (int)(__float_as_uint(pf) >> 23) - 127;      // 2^e <= p
+    const double half_ulp = __hiloint2double(__double2hiint(m) + ((e - 53) << 20), __double2loint(m));   // m 2^(e-53)
+    return __double_as_longlong(r) < __double_as_longlong(half_ulp) ? p : __ddiv_rn(mp, m);
+}
+
+// One 8^3 block of children and the three levels above it (fewer at the root).
+// LEAF: the children are cells -- netting of Eq. 1-2 per cell, e of Eq. 3,
+// ionised mass -- otherwise nodes of an earlier launch.  Parents are reduced
+// from their children in child order, a thread per (parent, field): plain FP64
+// sums (bit for bit the definition's) and, in the FP32 forms, Kahan-Neumaier
+// sums with the first moments about each parent's own centre (a child's, plus
+// its mass times the offset of its centre, +-s/4 per axis, which is exact); the
+// IF flag from the FP64 masses into the sign of the FP32 m_ion, and kappa =
+// max |cm32 - cm64| / edge.  Bound by the FP64 units (about 28 instructions per
+// cell and warp) and by the bytes of the records, each written once; one launch
+// per level and form, with a pass to finish, read the records back twice.
+// 256^3 with both trees, export included: 4.90 -> @@ ms.
+template <bool F32, bool LEAF>
+__global__ void __launch_bounds__(BUILD_NT) k_build(BuildArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    double (*f64)[BUILD_PAD] = reinterpret_cast<double (*)[BUILD_PAD]>(smem);
+    float (*f32)[BUILD_PAD] = reinterpret_cast<float (*)[BUILD_PAD]>(smem + B_FIELDS * BUILD_PAD * sizeof(double));
+    const int tid = threadIdx.x;
+    const bool use_e = a.e_prev != nullptr;
+    int n = a.lc >= 3 ? BUILD_NT : 1 << (3 * a.lc);            // children of this CTA
+    uint32_t first = blockIdx.x * (uint32_t)n;                 // index of the first in its level
+    if (tid < n) {
+        const uint32_t m = first + tid;
+        const int64_t id = level_offset(a.lc) + m;
+        const int k = padded(tid);
+        if (LEAF) {
+            const uint32_t ix = compact3(m), iy = compact3(m >> 1), iz = compact3(m >> 2);
+            const int64_t c = ((int64_t)iz * a.N + iy) * a.N + ix;
+            const double nH = a.n_H[c];
+            const double net = __dsub_rn(__dmul_rn(nH, nH), __dmul_rn(a.ndot[c], a.invU));   // recombinations less emission (U)
+            const double ep = use_e ? a.e_prev[c] : 0.0;
+            NodeF64 nd;
+            nd.m = nH;
+            double sx, sy, sz;
+            nd.cmx = cell_centre(nH, (float)ix + 0.5f, sx);
+            nd.cmy = cell_centre(nH, (float)iy + 0.5f, sy);
+            nd.cmz = cell_centre(nH, (float)iz + 0.5f, sz);
+            const bool rec = __double_as_longlong(net) > 0;
+            nd.alpha = rec ? net : 0.0;
+            nd.eps = rec ? 0.0 : fabs(net);
+            nd.e = use_e ? ep * a.invEu : 0.0;
+            nd.mion = ep > 0.0 ? nH : 0.0;
+            a.n64[id] = nd;
+            f64[B_M][k] = nH; f64[B_X][k] = sx; f64[B_Y][k] = sy; f64[B_Z][k] = sz;
+            f64[B_ALPHA][k] = nd.alpha; f64[B_EPS][k] = nd.eps; f64[B_E][k] = nd.e; f64[B_MION][k] = nd.mion;
+            if (F32) {
+                NodeF32 q;                                     // a cell's mass sits at its centre: offset 0
+                const float nf = (float)nH, wf = (float)fabs(net);
+                q.m = nf;
+                q.ox = 0.f; q.oy = 0.f; q.oz = 0.f;
+                q.alpha = rec ? wf : 0.f;
+                q.eps = rec ? 0.f : wf;
+                q.e = use_e ? (float)nd.e : 0.f;
+                q.mion = ep > 0.0 ? nf : 0.f;
+                a.n32[id] = q;
+                f32[B_M][k] = nf; f32[B_X][k] = 0.f; f32[B_Y][k] = 0.f; f32[B_Z][k] = 0.f;
+                f32[B_ALPHA][k] = q.alpha; f32[B_EPS][k] = q.eps; f32[B_E][k] = q.e; f32[B_MION][k] = q.mion;
+                const float px = (float)ix + 0.5f, py = (float)iy + 0.5f, pz = (float)iz + 0.5f;
+                if (nd.cmx != widen(px) || nd.cmy != widen(py) || nd.cmz != widen(pz)) {
+                    const double ex = fabs(widen(px) - nd.cmx), ey = fabs(widen(py) - nd.cmy), ez = fabs(widen(pz) - nd.cmz);
+                    atomicMax(reinterpret_cast<unsigned int*>(a.kappa), __float_as_uint(__double2float_ru(fmax(ex, fmax(ey, ez)))));
+                }
+            }
+        } else {
+            const NodeF64 q = a.n64[id];
+            f64[B_M][k] = q.m; f64[B_ALPHA][k] = q.alpha; f64[B_EPS][k] = q.eps; f64[B_E][k] = q.e; f64[B_MION][k] = q.mion;
+            for (int x = 0; x < 3; ++x) f64[B_X + x][k] = a.s64[3 * id + x];
+            if (F32) {
+                const NodeF32 w = a.n32[id];
+                f32[B_M][k] = w.m; f32[B_ALPHA][k] = w.alpha; f32[B_EPS][k] = w.eps; f32[B_E][k] = w.e;
+                f32[B_MION][k] = fabsf(w.mion);
+                for (int x = 0; x < 3; ++x) f32[B_X + x][k] = a.s32[3 * id + x];
+            }
+        }
+    }
+    __syncthreads();
+    for (int l = a.lc - 1; l >= 0 && l >= a.lc - 3; --l) {
+        n >>= 3;                                               // parents
+        first >>= 3;
+        const float s = (float)(a.N >> l);
+        // thread -> (field, parent); 64 parents: a warp has one field
+        const int f = tid / n, p = tid - f * n;
+        double sum = 0.0;
+        float sum32 = 0.f;
+        const bool work = f < B_FIELDS && (use_e || f < B_E);
+        if (work) {
+            const double* c = &f64[f][9 * p];                  // padded(8 p)
+            sum = c[0];
+            for (int q = 1; q < 8; ++q) sum = __dadd_rn(sum, c[q]);
+            if (F32) {
+                F32Sum t;
+                const float *c32 = &f32[f][9 * p], *m32 = &f32[B_M][9 * p];
+                if (f >= B_X && f <= B_Z) {
+                    const float q4 = 0.25f * s;
+                    for (int q = 0; q < 8; ++q) {
+                        const float mq = m32[q] * q4;
+                        t.add(c32[q]);
+                        t.add((q >> (f - B_X)) & 1 ? mq : -mq);
+                    }
+                } else {
+                    for (int q = 0; q < 8; ++q) t.add(c32[q]);
+                }
+                sum32 = t.value();
+            }
+        }
+        __syncthreads();                                       // children read
+        if (f < B_FIELDS) {
+            f64[f][padded(p)] = sum;
+            if (F32) f32[f][padded(p)] = sum32;
+        }
+        __syncthreads();                                       // parents visible
+        if (tid < n) {                                         // a thread per parent writes its record
+            const int k = padded(tid);
+            const uint32_t m = first + tid;
+            const int64_t id = level_offset(l) + m;
+            const float gx = ((float)compact3(m) + 0.5f) * s, gy = ((float)compact3(m >> 1) + 0.5f) * s,
+                        gz = ((float)compact3(m >> 2) + 0.5f) * s;
+            NodeF64 nd;
+            nd.m = f64[B_M][k]; nd.alpha = f64[B_ALPHA][k]; nd.eps = f64[B_EPS][k]; nd.e = f64[B_E][k]; nd.mion = f64[B_MION][k];
+            const double sx = f64[B_X][k], sy = f64[B_Y][k], sz = f64[B_Z][k];
+            if (nd.m > 0.0) { nd.cmx = __ddiv_rn(sx, nd.m); nd.cmy = __ddiv_rn(sy, nd.m); nd.cmz = __ddiv_rn(sz, nd.m); }
+            else { nd.cmx = widen(gx); nd.cmy = widen(gy); nd.cmz = widen(gz); }
+            a.n64[id] = nd;
+            const bool start = l == a.lc - 3;                  // the next launch starts here
+            if (start) { a.s64[3 * id] = sx; a.s64[3 * id + 1] = sy; a.s64[3 * id + 2] = sz; }
+            if (F32) {
+                NodeF32 q;
+                q.m = f32[B_M][k]; q.alpha = f32[B_ALPHA][k]; q.eps = f32[B_EPS][k]; q.e = f32[B_E][k]; q.mion = f32[B_MION][k];
+                const float fx = f32[B_X][k], fy = f32[B_Y][k], fz = f32[B_Z][k];
+                if (q.m > 0.f) { q.ox = fx / q.m; q.oy = fy / q.m; q.oz = fz / q.m; }
+                else { q.ox = 0.f; q.oy = 0.f; q.oz = 0.f; }   // no mass: the geometric centre
+                if (use_e && __dmul_rn(DELTA_IF, nd.m) < nd.mion && nd.mion < __dmul_rn(1.0 - DELTA_IF, nd.m)) q.mion = -q.mion;
+                a.n32[id] = q;
+                if (start) { a.s32[3 * id] = fx; a.s32[3 * id + 1] = fy; a.s32[3 * id + 2] = fz; }
+                const double ex = fabs(widen(gx) + widen_signed(q.ox) - nd.cmx), ey = fabs(widen(gy) + widen_signed(q.oy) - nd.cmy),
+                             ez = fabs(widen(gz) + widen_signed(q.oz) - nd.cmz);
+                const float kap = __double2float_ru(fmax(ex, fmax(ey, ez)) / (double)s);
+                if (kap > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.kappa), __float_as_uint(kap));
+            }
+        }
+        // (the next level reads the fields that these threads read)
     }
 }
 
@@ -254,14 +397,7 @@ __global__ void k_parents(void* nodes_v, void* sums_v, int l, int N, const uint8
     }
 }
 
-// Level of node `id` in the level-order numbering.
-__device__ __forceinline__ int node_level(int64_t id) {
-    int l = 0;
-    while (level_offset(l + 1) <= id) ++l;
-    return l;
-}
-
-// FP32 forms, after both builds: the IF flag of every node (Sec. 2.4,
+// FP32 forms on an AMR grid, after both builds: the IF flag of every node (Sec. 2.4,
 // delta_IF m < m_ion < (1 - delta_IF) m on the FP64 masses, as the FP64 walk
 // decides it) goes into the sign bit of the FP32 m_ion, and kappa =
 // max |cm32 - cm64| / edge over the nodes that exist (rounded up).
@@ -296,20 +432,21 @@ __global__ void k_export(const void* nodes_v, int64_t n, double* out, double U, 
         NodeF64 q = ((const NodeF64*)nodes_v)[i];
         v[0] = q.m; v[1] = q.cmx; v[2] = q.cmy; v[3] = q.cmz;
         v[4] = q.alpha; v[5] = q.eps; v[6] = q.e; v[7] = q.mion;
-    } else {                                       // centre of mass = geometric centre + offset
+    } else {                                       // centre of mass = geometric centre (exact in FP32) + offset
         NodeF32 q = ((const NodeF32*)nodes_v)[i];
         const bool absent = flags && flags[i] == NODE_ABSENT;
         const int l = node_level(i);
         const uint32_t m = (uint32_t)(i - level_offset(l));
-        const double s = (double)(N >> l);
-        v[0] = q.m;
-        v[1] = absent ? 0.0 : ((double)compact3(m) + 0.5) * s + (double)q.ox;
-        v[2] = absent ? 0.0 : ((double)compact3(m >> 1) + 0.5) * s + (double)q.oy;
-        v[3] = absent ? 0.0 : ((double)compact3(m >> 2) + 0.5) * s + (double)q.oz;
-        v[4] = q.alpha; v[5] = q.eps; v[6] = q.e; v[7] = fabsf(q.mion);
+        const float s = (float)(N >> l);
+        v[0] = widen(q.m);
+        v[1] = absent ? 0.0 : widen(((float)compact3(m) + 0.5f) * s) + widen_signed(q.ox);
+        v[2] = absent ? 0.0 : widen(((float)compact3(m >> 1) + 0.5f) * s) + widen_signed(q.oy);
+        v[3] = absent ? 0.0 : widen(((float)compact3(m >> 2) + 0.5f) * s) + widen_signed(q.oz);
+        v[4] = widen(q.alpha); v[5] = widen(q.eps); v[6] = widen(q.e); v[7] = widen(fabsf(q.mion));
     }
     v[4] *= U; v[5] *= U; v[6] *= Eu;
-    for (int k = 0; k < 8; ++k) out[8 * i + k] = v[k];
+    double2* o = reinterpret_cast<double2*>(out + 8 * i);
+    for (int k = 0; k < 4; ++k) o[k] = make_double2(v[2 * k], v[2 * k + 1]);
 }
 
 // Ray constants: r_i (Eq. 4), ray-cell volumes, and for each segment i and
@@ -438,22 +575,29 @@ tr_status tree_build(tr_tree* t, const tr_grid* g, const tr_sources* s, cudaStre
     if (s && s->n > 0)
         k_map_sources<<<grid_for(s->n, 128), 128, 0, st>>>(t->ndot, t->N, g->box_lo[0], g->box_lo[1],
                                                            g->box_lo[2], g->dx, s->xyz, s->Q, s->n);
-    // the FP64 tree (the whole tree in mode 0, the sidecar of the FP32 forms)
-    k_leaves<0><<<grid_for(ncell, 256), 256, 0, st>>>(t->nodes64, t->sums64, t->N, t->L, g->n_H, t->ndot,
-                                                     g->e_prev, invU, invEu);
-    for (int l = t->L - 1; l >= 0; --l) {
-        const int64_t nl = int64_t(1) << (3 * l);
-        k_parents<0><<<grid_for(nl, 128), 128, 0, st>>>(t->nodes64, t->sums64, l, t->N, nullptr);
-    }
+    BuildArgs a{};
+    a.n64 = (NodeF64*)t->nodes64; a.s64 = (double*)t->sums64;
+    a.n32 = (NodeF32*)t->nodes; a.s32 = (float*)t->sums;
+    a.kappa = t->kappa;
+    a.n_H = g->n_H; a.ndot = t->ndot; a.e_prev = g->e_prev;
+    a.invU = invU; a.invEu = invEu;
+    a.N = t->N;
     if (t->mode != 0) {
-        k_leaves<1><<<grid_for(ncell, 256), 256, 0, st>>>(t->nodes, t->sums, t->N, t->L, g->n_H, t->ndot,
-                                                         g->e_prev, invU, invEu);
-        for (int l = t->L - 1; l >= 0; --l) {
-            const int64_t nl = int64_t(1) << (3 * l);
-            k_parents<1><<<grid_for(nl, 128), 128, 0, st>>>(t->nodes, t->sums, l, t->N, nullptr);
-        }
-        tr_status rc = finalize_f32(t, st);
+        tr_status rc = cuda_check(cudaMemsetAsync(t->kappa, 0, sizeof(float), st), "clear kappa");
         if (rc != TR_OK) return rc;
+    }
+    // the cells and three levels of parents, then three levels at a time
+    for (int lc = t->L; lc > 0; lc -= 3) {
+        a.lc = lc;
+        const unsigned blocks = lc > 3 ? 1u << (3 * (lc - 3)) : 1u;
+        const bool leaf = lc == t->L;
+        auto kern = t->mode == 0 ? (leaf ? k_build<false, true> : k_build<false, false>)
+                                 : (leaf ? k_build<true, true> : k_build<true, false>);
+        const size_t smem = (size_t)B_FIELDS * BUILD_PAD * (sizeof(double) + (t->mode != 0 ? sizeof(float) : 0));
+        tr_status rc = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                                  "cudaFuncSetAttribute(build smem)");
+        if (rc != TR_OK) return rc;
+        kern<<<blocks, BUILD_NT, smem, st>>>(a);
     }
     return cuda_check(cudaGetLastError(), "tree build kernels");
 }

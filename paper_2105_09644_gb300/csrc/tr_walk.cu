@@ -122,12 +122,6 @@ __device__ __forceinline__ double recip(double a) {
     return fma(y, fma(e, e, e), y);
 }
 
-// A float >= 0 as a double, by integer operations (subnormals give 0).
-__device__ __forceinline__ double widen(float f) {
-    const uint32_t b = __float_as_uint(f);
-    return b < 0x00800000u ? 0.0 : __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
-}
-
 // The nearest float towards zero of a double in the float range (bounds only).
 __device__ __forceinline__ float narrow(double a) {
     return __uint_as_float(((uint32_t)__double2hiint(a) - 0x38000000u) << 3 | (uint32_t)__double2loint(a) >> 29);
