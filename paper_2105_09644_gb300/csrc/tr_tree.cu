@@ -99,16 +99,20 @@ __device__ __forceinline__ double cell_centre(double m, float pf, double& mp) {
 // sums with the first moments about each parent's own centre (a child's, plus
 // its mass times the offset of its centre, +-s/4 per axis, which is exact); the
 // IF flag from the FP64 masses into the sign of the FP32 m_ion, and kappa =
-// max |cm32 - cm64| / edge.  Bound by the FP64 units (about 28 instructions per
-// cell and warp) and by the bytes of the records, each written once; one launch
-// per level and form, with a pass to finish, read the records back twice.
-// 256^3 with both trees, export included: 4.90 -> 3.04 ms.
+// max |cm32 - cm64| / edge, one atomic per CTA (one per parent: 3.04 ms for the
+// figure below).  Bound by the FP64 units and by the latency of the three
+// levels; each record is written once, where one launch per level and form
+// with a pass to finish read them back twice.  256^3 with both trees, export
+// included: 4.90 -> 2.40 ms.
 template <bool F32, bool LEAF>
-__global__ void __launch_bounds__(BUILD_NT) k_build(BuildArgs a) {
+__global__ void __launch_bounds__(BUILD_NT, 3) k_build(BuildArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     double (*f64)[BUILD_PAD] = reinterpret_cast<double (*)[BUILD_PAD]>(smem);
     float (*f32)[BUILD_PAD] = reinterpret_cast<float (*)[BUILD_PAD]>(smem + B_FIELDS * BUILD_PAD * sizeof(double));
     const int tid = threadIdx.x;
+    __shared__ unsigned s_kap;
+    float kap = 0.f;
+    if (tid == 0) s_kap = 0u;
     const bool use_e = a.e_prev != nullptr;
     int n = a.lc >= 3 ? BUILD_NT : 1 << (3 * a.lc);            // children of this CTA
     uint32_t first = blockIdx.x * (uint32_t)n;                 // index of the first in its level
@@ -132,7 +136,8 @@ __global__ void __launch_bounds__(BUILD_NT) k_build(BuildArgs a) {
             nd.alpha = rec ? net : 0.0;
             nd.eps = rec ? 0.0 : fabs(net);
             nd.e = use_e ? ep * a.invEu : 0.0;
-            nd.mion = ep > 0.0 ? nH : 0.0;
+            const bool lit = __double_as_longlong(ep) > 0;
+            nd.mion = lit ? nH : 0.0;
             a.n64[id] = nd;
             f64[B_M][k] = nH; f64[B_X][k] = sx; f64[B_Y][k] = sy; f64[B_Z][k] = sz;
             f64[B_ALPHA][k] = nd.alpha; f64[B_EPS][k] = nd.eps; f64[B_E][k] = nd.e; f64[B_MION][k] = nd.mion;
@@ -144,14 +149,15 @@ __global__ void __launch_bounds__(BUILD_NT) k_build(BuildArgs a) {
                 q.alpha = rec ? wf : 0.f;
                 q.eps = rec ? 0.f : wf;
                 q.e = use_e ? (float)nd.e : 0.f;
-                q.mion = ep > 0.0 ? nf : 0.f;
+                q.mion = lit ? nf : 0.f;
                 a.n32[id] = q;
                 f32[B_M][k] = nf; f32[B_X][k] = 0.f; f32[B_Y][k] = 0.f; f32[B_Z][k] = 0.f;
                 f32[B_ALPHA][k] = q.alpha; f32[B_EPS][k] = q.eps; f32[B_E][k] = q.e; f32[B_MION][k] = q.mion;
                 const float px = (float)ix + 0.5f, py = (float)iy + 0.5f, pz = (float)iz + 0.5f;
-                if (nd.cmx != widen(px) || nd.cmy != widen(py) || nd.cmz != widen(pz)) {
+                auto differs = [](double u, double v) { return __double_as_longlong(u) != __double_as_longlong(v); };
+                if (differs(nd.cmx, widen(px)) || differs(nd.cmy, widen(py)) || differs(nd.cmz, widen(pz))) {
                     const double ex = fabs(widen(px) - nd.cmx), ey = fabs(widen(py) - nd.cmy), ez = fabs(widen(pz) - nd.cmz);
-                    atomicMax(reinterpret_cast<unsigned int*>(a.kappa), __float_as_uint(__double2float_ru(fmax(ex, fmax(ey, ez)))));
+                    kap = __double2float_ru(fmax(ex, fmax(ey, ez)));
                 }
             }
         } else {
@@ -197,41 +203,53 @@ __global__ void __launch_bounds__(BUILD_NT) k_build(BuildArgs a) {
             }
         }
         __syncthreads();                                       // children read
+        const int k = padded(p);
         if (f < B_FIELDS) {
-            f64[f][padded(p)] = sum;
-            if (F32) f32[f][padded(p)] = sum32;
+            f64[f][k] = sum;
+            if (F32) f32[f][k] = sum32;
         }
         __syncthreads();                                       // parents visible
-        if (tid < n) {                                         // a thread per parent writes its record
-            const int k = padded(tid);
-            const uint32_t m = first + tid;
+        if (f < B_FIELDS) {                                    // each thread writes its field of the records
+            const uint32_t m = first + p;
             const int64_t id = level_offset(l) + m;
-            const float gx = ((float)compact3(m) + 0.5f) * s, gy = ((float)compact3(m >> 1) + 0.5f) * s,
-                        gz = ((float)compact3(m >> 2) + 0.5f) * s;
-            NodeF64 nd;
-            nd.m = f64[B_M][k]; nd.alpha = f64[B_ALPHA][k]; nd.eps = f64[B_EPS][k]; nd.e = f64[B_E][k]; nd.mion = f64[B_MION][k];
-            const double sx = f64[B_X][k], sy = f64[B_Y][k], sz = f64[B_Z][k];
-            if (nd.m > 0.0) { nd.cmx = __ddiv_rn(sx, nd.m); nd.cmy = __ddiv_rn(sy, nd.m); nd.cmz = __ddiv_rn(sz, nd.m); }
-            else { nd.cmx = widen(gx); nd.cmy = widen(gy); nd.cmz = widen(gz); }
-            a.n64[id] = nd;
             const bool start = l == a.lc - 3;                  // the next launch starts here
-            if (start) { a.s64[3 * id] = sx; a.s64[3 * id + 1] = sy; a.s64[3 * id + 2] = sz; }
-            if (F32) {
-                NodeF32 q;
-                q.m = f32[B_M][k]; q.alpha = f32[B_ALPHA][k]; q.eps = f32[B_EPS][k]; q.e = f32[B_E][k]; q.mion = f32[B_MION][k];
-                const float fx = f32[B_X][k], fy = f32[B_Y][k], fz = f32[B_Z][k];
-                if (q.m > 0.f) { q.ox = fx / q.m; q.oy = fy / q.m; q.oz = fz / q.m; }
-                else { q.ox = 0.f; q.oy = 0.f; q.oz = 0.f; }   // no mass: the geometric centre
-                if (use_e && __dmul_rn(DELTA_IF, nd.m) < nd.mion && nd.mion < __dmul_rn(1.0 - DELTA_IF, nd.m)) q.mion = -q.mion;
-                a.n32[id] = q;
-                if (start) { a.s32[3 * id] = fx; a.s32[3 * id + 1] = fy; a.s32[3 * id + 2] = fz; }
-                const double ex = fabs(widen(gx) + widen_signed(q.ox) - nd.cmx), ey = fabs(widen(gy) + widen_signed(q.oy) - nd.cmy),
-                             ez = fabs(widen(gz) + widen_signed(q.oz) - nd.cmz);
-                const float kap = __double2float_ru(fmax(ex, fmax(ey, ez)) / (double)s);
-                if (kap > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.kappa), __float_as_uint(kap));
+            double* r64 = reinterpret_cast<double*>(a.n64 + id);
+            float* r32 = reinterpret_cast<float*>(a.n32 + id);
+            if (f >= B_X && f <= B_Z) {
+                const int x = f - B_X;
+                const float g = ((float)compact3(m >> x) + 0.5f) * s;   // the geometric centre, exact
+                const double m64 = f64[B_M][k];
+                const double cm = m64 > 0.0 ? __ddiv_rn(sum, m64) : widen(g);
+                r64[x] = cm;
+                if (start) a.s64[3 * id + x] = sum;
+                if (F32) {
+                    const float mf = f32[B_M][k], o = mf > 0.f ? sum32 / mf : 0.f;
+                    r32[x] = o;
+                    if (start) a.s32[3 * id + x] = sum32;
+                    const double ex = fabs(widen(g) + widen_signed(o) - cm) * widen(1.f / s);   // (s a power of two)
+                    kap = fmaxf(kap, __double2float_ru(ex));
+                }
+            } else {
+                const int at = f == B_M ? 3 : f;               // record order: cm, m, alpha, eps, e, mion
+                r64[at] = sum;
+                if (F32) {
+                    float v = sum32;
+                    if (f == B_MION && use_e) {
+                        const double m64 = f64[B_M][k];
+                        if (__dmul_rn(DELTA_IF, m64) < sum && sum < __dmul_rn(1.0 - DELTA_IF, m64)) v = -v;
+                    }
+                    r32[at] = v;
+                }
             }
         }
         // (the next level reads the fields that these threads read)
+    }
+    if (F32) {                                                 // one atomic per CTA that raises kappa
+        const unsigned v = __reduce_max_sync(0xffffffffu, __float_as_uint(kap));
+        if ((tid & 31) == 0 && v) atomicMax(&s_kap, v);
+        __syncthreads();
+        if (tid == 0 && s_kap > __ldcg(reinterpret_cast<const unsigned int*>(a.kappa)))
+            atomicMax(reinterpret_cast<unsigned int*>(a.kappa), s_kap);
     }
 }
 
