@@ -223,9 +223,10 @@ tr_status tr_ray_sweep(const tr_rays* r, double* F_out, double* e_out, uint8_t* 
 tr_status tr_walk_sweep(const tr_tree* t, double* F_out, double* e_out, uint8_t* ion_out,
                         tr_stream stream);
 
-/* Continuous batching of independent problems: ONE persistent launch walks,
- * maps and sweeps the targets of several built trees (different grid sizes,
- * sources and N_PIX allowed; one precision per batch).  For tree i it does
+/* Continuous batching of independent problems: persistent launches, one for
+ * each size class of ray bins among them, walk, map and sweep the targets of
+ * several built trees (different grid sizes, sources and N_PIX allowed; one
+ * precision per batch).  For tree i it does
  * the cells whose Morton index (x bit 0, y bit 1, z bit 2 of each triple)
  * lies in [first[i], first[i] + count[i]), writing F_out[i], e_out[i] and
  * ion_out[i] at the cells' C-order indices (device arrays of that tree's

@@ -2103,6 +2103,26 @@ tr_status launch_jobs(int mode, int out, bool var, size_t smem, const WalkArgs* 
                : launch_jobs_v<false>(mode, out, smem, jobs, job_end, n_jobs, total, counter, st);
 }
 
+// Targets that an SM holds at once in the fused walk of a form.
+template <int MODE>
+int targets_per_sm_m(size_t smem) {
+    constexpr int F = OUT_FUSED;
+    const int w128 = resident_warps<128>(k_walk<MODE, F, 128, 5, false>, smem), w256 = resident_warps<256>(k_walk<MODE, F, 256, 2, false>, smem);
+    int best = w128, per = w128 / 4;
+    if constexpr (MODE != 0) {
+        const int w6 = resident_warps<128>(k_walk<MODE, F, 128, 6, false>, smem);
+        if (w6 > best) { best = w6; per = w6 / 4; }
+    }
+    if (w256 > best) { best = w256; per = w256 / 8; }
+    if constexpr (MODE != 0)
+        if (resident_warps<512>(k_walk<MODE, F, 512, 1, false>, smem) > best) per = 1;
+    return per;
+}
+int targets_per_sm(int mode, size_t smem) {
+    return mode == 0 ? targets_per_sm_m<0>(smem) : (mode == 1 ? targets_per_sm_m<1>(smem) : targets_per_sm_m<2>(smem));
+}
+constexpr int BATCH_WAVES = 4;              // targets per resident target below which a batch's group is too small
+
 bool uses_variants(const tr_tree* t) {
     return t->p.kernel_alpha != TR_KERNEL_WP || t->p.kernel_eps != TR_EPS_WF3 || t->p.bc != TR_BC_ISOLATED;
 }
@@ -2162,33 +2182,59 @@ tr_status cd_run(const tr_tree* t, const int64_t* targets, int64_t n_targets, do
 tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, const int64_t* count, int n,
                          double* const* F, double* const* e, uint8_t* const* ion, void* jobbuf, unsigned int* counter,
                          cudaStream_t st) {
+    // Jobs by the number of targets that an SM holds at once with each tree's
+    // own ray bins, one launch for each: a tree with N_PIX 192 would otherwise
+    // set the shared memory, and so the warps per SM, of every target (two 64^3
+    // and two 32^3 trees, one with N_PIX 192: 141 -> 75 ms).  A group too small
+    // to fill the GPU a few times over joins the next with larger bins.
+    struct Item { int tree, per_sm; size_t smem; };
+    const int mode = trees[0]->mode;
+    std::vector<Item> items;
+    for (int i = 0; i < n; ++i)
+        if (count[i] > 0) {
+            const size_t m = walk_smem(trees[i]);
+            items.push_back({i, targets_per_sm(mode, m), m});
+        }
+    std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.per_sm > y.per_sm; });
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     std::vector<unsigned char> host(walk_job_bytes(n));
     WalkArgs* hj = reinterpret_cast<WalkArgs*>(host.data());
     int64_t* he = reinterpret_cast<int64_t*>(host.data() + (size_t)n * sizeof(WalkArgs));
-    size_t smem = 0;
-    int64_t total = 0;
-    bool var = false;
+    struct Group { int first, n; size_t smem; int64_t total; bool var; };
+    std::vector<Group> groups;
     tr_status s = TR_OK;
-    for (int i = 0; i < n; ++i) {
-        var = var || uses_variants(trees[i]);
+    for (int k = 0; k < (int)items.size(); ++k) {
+        const int i = items[k].tree;
+        const bool join = k > 0 && (items[k].per_sm == items[k - 1].per_sm ||
+                                    groups.back().total < (int64_t)sms * items[k - 1].per_sm * BATCH_WAVES);
+        if (!join) groups.push_back({k, 0, 0, 0, false});
+        Group& g = groups.back();
         WalkArgs a = make_args(trees[i]);
         a.targets = nullptr;
         a.first = first[i];
         a.n_targets = count[i];
         a.F = F ? F[i] : nullptr; a.E = e ? e[i] : nullptr; a.ion = ion ? ion[i] : nullptr;
-        hj[i] = a;
-        total += count[i];
-        he[i] = total;
-        smem = std::max(smem, walk_smem(trees[i]));
+        hj[k] = a;
+        ++g.n;
+        g.total += count[i];
+        he[k] = g.total;
+        g.smem = std::max(g.smem, items[k].smem);
+        g.var = g.var || uses_variants(trees[i]);
+    }
+    for (int i = 0; i < n; ++i) {
         if (s == TR_OK) s = cuda_check(cudaMemsetAsync(trees[i]->status, 0, 4 * sizeof(int32_t), st), "status reset");
         if (s == TR_OK) s = cuda_check(cudaMemsetAsync(trees[i]->stats, 0, N_STATS * sizeof(unsigned long long), st), "stats reset");
     }
     if (s == TR_OK) s = cuda_check(cudaMemcpyAsync(jobbuf, host.data(), host.size(), cudaMemcpyHostToDevice, st), "job copy");
     if (s == TR_OK) s = cuda_check(cudaStreamSynchronize(st), "job copy");
-    if (s != TR_OK || total == 0) return s;
     const WalkArgs* jobs = reinterpret_cast<const WalkArgs*>(jobbuf);
     const int64_t* job_end = reinterpret_cast<const int64_t*>(reinterpret_cast<unsigned char*>(jobbuf) + (size_t)n * sizeof(WalkArgs));
-    return launch_jobs(trees[0]->mode, OUT_FUSED, var, smem, jobs, job_end, n, total, counter, st);
+    for (const Group& g : groups)
+        if (s == TR_OK)
+            s = launch_jobs(mode, OUT_FUSED, g.var, g.smem, jobs + g.first, job_end + g.first, g.n, g.total, counter, st);
+    return s;
 }
 
 tr_status sweep_run(const tr_rays* r, double* F, double* e, uint8_t* ion, cudaStream_t st) {
