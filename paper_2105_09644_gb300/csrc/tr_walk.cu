@@ -32,7 +32,6 @@
 // without radial points, and a separate instantiation for non-default
 // kernels and boundaries.
 #include <algorithm>
-#include <cstring>
 #include <vector>
 
 #include "tr_internal.cuh"
@@ -1961,6 +1960,29 @@ __global__ void __launch_bounds__(NT) k_sweep_stored(WalkArgs a, const double* b
 
 constexpr int SWEEP_NT = 128;               // threads per target of the stored-bins sweep
 
+// Before a walk of one tree: its job record (passed as the kernel's parameter,
+// so that no host buffer has to outlive the call), its status words and
+// counters cleared, and the work counter.  One launch in place of three
+// clears, a copy and a wait for the copy (16^3 solve 281 -> 267 us).
+__global__ void __launch_bounds__(128) k_job_start(const __grid_constant__ WalkArgs a, int64_t end, WalkArgs* job, int64_t* job_end,
+                                                   unsigned int* counter) {
+    const int* src = reinterpret_cast<const int*>(&a);
+    for (int k = threadIdx.x; k < (int)(sizeof(WalkArgs) / sizeof(int)); k += 128) reinterpret_cast<int*>(job)[k] = src[k];
+    if (threadIdx.x < 4) a.status[threadIdx.x] = 0;
+    if (threadIdx.x < N_STATS) a.stats[threadIdx.x] = 0ull;
+    if (threadIdx.x == 0) { *job_end = end; *counter = 0u; }
+}
+
+tr_status job_start(const WalkArgs& a, const tr_tree* t, int64_t n_targets, const WalkArgs** jobs, const int64_t** job_end,
+                    cudaStream_t st) {
+    WalkArgs* j = reinterpret_cast<WalkArgs*>(t->jobbuf);
+    int64_t* e = reinterpret_cast<int64_t*>(reinterpret_cast<unsigned char*>(t->jobbuf) + sizeof(WalkArgs));
+    k_job_start<<<1, 128, 0, st>>>(a, n_targets, j, e, t->counter);
+    *jobs = j;
+    *job_end = e;
+    return cuda_check(cudaGetLastError(), "job record kernel");
+}
+
 size_t walk_smem(const tr_tree* t) {
     const int nq = t->use_e ? 3 : 2;
     return (size_t)nq * t->npix * t->nr * 8 + (size_t)STACK_CAP * 4;
@@ -2011,8 +2033,6 @@ tr_status launch_persistent(K kernel, size_t smem, const WalkArgs* jobs, const i
     s = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem), "occupancy query");
     if (s != TR_OK) return s;
     if (per_sm < 1) return set_error(TR_EUNSUPPORTED, "ray bins need %zu bytes of shared memory per target", smem);
-    s = cuda_check(cudaMemsetAsync(counter, 0, sizeof(unsigned int), st), "counter reset");
-    if (s != TR_OK) return s;
     int64_t blocks = (int64_t)sms * per_sm;
     if (blocks > total) blocks = total > 0 ? total : 1;
     kernel<<<(unsigned)blocks, NT, smem, st>>>(jobs, job_end, n_jobs, counter);
@@ -2141,18 +2161,10 @@ tr_status walk_run(const tr_tree* t, const int64_t* targets, int64_t n_targets, 
     a.bins_out = out.bins; a.ids_out = out.ids; a.counts_out = out.counts; a.eps_self_out = out.eps_self;
     a.scales_out = out.scales;
     a.acc_cap = out.acc_cap;
-    // the job record goes to the tree's job buffer; the copy completes before
-    // return (host staging), so the stack record may go away afterwards
-    unsigned char host[sizeof(WalkArgs) + sizeof(int64_t)];
-    memcpy(host, &a, sizeof(WalkArgs));
-    memcpy(host + sizeof(WalkArgs), &n_targets, sizeof(int64_t));
-    tr_status s = cuda_check(cudaMemsetAsync(t->status, 0, 4 * sizeof(int32_t), st), "status reset");
-    if (s == TR_OK) s = cuda_check(cudaMemsetAsync(t->stats, 0, N_STATS * sizeof(unsigned long long), st), "stats reset");
-    if (s == TR_OK) s = cuda_check(cudaMemcpyAsync(t->jobbuf, host, sizeof host, cudaMemcpyHostToDevice, st), "job copy");
-    if (s == TR_OK) s = cuda_check(cudaStreamSynchronize(st), "job copy");
+    const WalkArgs* jobs = nullptr;
+    const int64_t* job_end = nullptr;
+    const tr_status s = job_start(a, t, n_targets, &jobs, &job_end, st);
     if (s != TR_OK || n_targets <= 0) return s;
-    const WalkArgs* jobs = reinterpret_cast<const WalkArgs*>(t->jobbuf);
-    const int64_t* job_end = reinterpret_cast<const int64_t*>(reinterpret_cast<const unsigned char*>(t->jobbuf) + sizeof(WalkArgs));
     return launch_jobs(t->mode, dump ? OUT_DUMP : OUT_FUSED, uses_variants(t), walk_smem(t), jobs, job_end, 1, n_targets,
                        t->counter, st);
 }
@@ -2165,16 +2177,10 @@ tr_status cd_run(const tr_tree* t, const int64_t* targets, int64_t n_targets, do
     a.cd_out = out;
     a.cd_conv = t->dx;
     a.cd_omega = 4.0 * PI_D / (double)t->npix;
-    unsigned char host[sizeof(WalkArgs) + sizeof(int64_t)];
-    memcpy(host, &a, sizeof(WalkArgs));
-    memcpy(host + sizeof(WalkArgs), &n_targets, sizeof(int64_t));
-    tr_status s = cuda_check(cudaMemsetAsync(t->status, 0, 4 * sizeof(int32_t), st), "status reset");
-    if (s == TR_OK) s = cuda_check(cudaMemsetAsync(t->stats, 0, N_STATS * sizeof(unsigned long long), st), "stats reset");
-    if (s == TR_OK) s = cuda_check(cudaMemcpyAsync(t->jobbuf, host, sizeof host, cudaMemcpyHostToDevice, st), "job copy");
-    if (s == TR_OK) s = cuda_check(cudaStreamSynchronize(st), "job copy");
+    const WalkArgs* jobs = nullptr;
+    const int64_t* job_end = nullptr;
+    const tr_status s = job_start(a, t, n_targets, &jobs, &job_end, st);
     if (s != TR_OK || n_targets <= 0) return s;
-    const WalkArgs* jobs = reinterpret_cast<const WalkArgs*>(t->jobbuf);
-    const int64_t* job_end = reinterpret_cast<const int64_t*>(reinterpret_cast<const unsigned char*>(t->jobbuf) + sizeof(WalkArgs));
     const size_t smem = (size_t)t->npix * 8 + (size_t)STACK_CAP * 4;
     return launch_jobs(t->mode, OUT_CD, uses_variants(t), smem, jobs, job_end, 1, n_targets, t->counter, st);
 }
@@ -2231,9 +2237,11 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
     if (s == TR_OK) s = cuda_check(cudaStreamSynchronize(st), "job copy");
     const WalkArgs* jobs = reinterpret_cast<const WalkArgs*>(jobbuf);
     const int64_t* job_end = reinterpret_cast<const int64_t*>(reinterpret_cast<unsigned char*>(jobbuf) + (size_t)n * sizeof(WalkArgs));
-    for (const Group& g : groups)
+    for (const Group& g : groups) {
+        if (s == TR_OK) s = cuda_check(cudaMemsetAsync(counter, 0, sizeof(unsigned int), st), "counter reset");
         if (s == TR_OK)
             s = launch_jobs(mode, OUT_FUSED, g.var, g.smem, jobs + g.first, job_end + g.first, g.n, g.total, counter, st);
+    }
     return s;
 }
 
