@@ -1201,13 +1201,19 @@ __device__ __forceinline__ double sweep_groups(const WalkArgs& a, const double* 
         const bool single = c == 1 && !bee;                   // zeta_s = zeta_d = 1 throughout
         const int wmax = __reduce_max_sync(FULL, (unsigned)w);
         const int itop = __reduce_max_sync(FULL, (unsigned)jtop);
-        float a_hi = in ? bin_value_f<1>(ba + itop, ia) * __ldg(a.inv_volf + itop) : 0.f;
+        auto alpha = [&](int i) { return in ? bin_value_f<1>(ba + i, ia) * __ldg(a.inv_volf + i) : 0.f; };
+        // the tables and the coefficient of a segment are fetched one segment
+        // ahead of the chain F_tot -> R -> Phi
+        const float* id2p = a.ID2f + (size_t)(itop - 1) * nr + jA;
+        const float* gp = (single ? a.Gf : a.GIf) + (size_t)(itop - 1) * nr + jA;
+        float a_hi = alpha(itop), a_nx = alpha(itop - 1), id2n = __ldg(id2p), gn = __ldg(gp);
         for (int i = itop - 1; i >= 0; --i) {
             if (!__any_sync(FULL, !sA)) break;                // every point of the warp spent
-            const float a_lo = in ? bin_value_f<1>(ba + i, ia) * __ldg(a.inv_volf + i) : 0.f;
+            const float a_lo = a_nx, id2 = id2n, g = gn;
+            if (i > 0) { id2p -= nr; gp -= nr; id2n = __ldg(id2p); gn = __ldg(gp); a_nx = alpha(i - 1); }
             const bool live = !sA && jA > i;
             const float ph = live ? phi_f(EA, LA) : 0.f;
-            float Fl = live ? ph * __ldg(a.ID2f + (size_t)i * nr + jA) : 0.f;   // Eq. 11 at the segment midpoint
+            float Fl = live ? ph * id2 : 0.f;                 // Eq. 11 at the segment midpoint
             for (int o = 1; o < wmax; o <<= 1) {
                 const float t = __shfl_xor_sync(FULL, Fl, o);
                 if (o < w) Fl += t;
@@ -1216,14 +1222,14 @@ __device__ __forceinline__ double sweep_groups(const WalkArgs& a, const double* 
                 const float A = a_lo + a_hi;                  // G carries the 1/2 of the mean
                 float R;
                 if (single) {
-                    R = A * __ldg(a.Gf + (size_t)i * nr + jA);                       // Eq. 14
+                    R = A * g;                                // Eq. 14
                 } else {
                     float zd = 1.f;                           // Eq. 17
                     if (bee) {
                         const float ev = bin_value_f<1>(bee + i + 1, ie) * __ldg(a.inv_volf + i + 1);
                         if (ev > 0.f) zd = fminf(2.f, __fdividef(Fl, ev));
                     }
-                    R = __fdividef(A * zd, Fl) * (__ldg(a.GIf + (size_t)i * nr + jA) * ph);   // zeta_s = F_j / Ftot
+                    R = __fdividef(A * zd, Fl) * (g * ph);    // zeta_s = F_j / Ftot
                 }
                 const float2 t = two_sum(LA.x, R);            // compensated L += R
                 const float2 Ln = two_sum(t.x, t.y + LA.y);
