@@ -8,7 +8,7 @@ over time.  The loop
   fit yet);
 * builds an admitted request's tree once and keeps it resident until the
   request is done;
-* launches ONE persistent walk kernel (tr_walk_sweep_batch) at a time over
+* makes ONE batched walk call (tr_walk_sweep_batch) at a time over
   a slice of the remaining target cells of every active request: requests
   with the least remaining work get their slice first, large requests are cut
   into Morton ranges so that they do not hold up small ones; while it runs,
