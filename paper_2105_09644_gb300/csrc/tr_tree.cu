@@ -463,8 +463,12 @@ __global__ void k_export(const void* nodes_v, int64_t n, double* out, double U, 
         v[4] = widen(q.alpha); v[5] = widen(q.eps); v[6] = widen(q.e); v[7] = widen(fabsf(q.mion));
     }
     v[4] *= U; v[5] *= U; v[6] *= Eu;
-    double2* o = reinterpret_cast<double2*>(out + 8 * i);
-    for (int k = 0; k < 4; ++k) o[k] = make_double2(v[2 * k], v[2 * k + 1]);
+    if ((reinterpret_cast<uintptr_t>(out) & 15) == 0) {        // the caller's array need only be aligned to doubles
+        double2* o = reinterpret_cast<double2*>(out + 8 * i);
+        for (int k = 0; k < 4; ++k) o[k] = make_double2(v[2 * k], v[2 * k + 1]);
+    } else {
+        for (int k = 0; k < 8; ++k) out[8 * i + k] = v[k];
+    }
 }
 
 // Ray constants: r_i (Eq. 4), ray-cell volumes, and for each segment i and
