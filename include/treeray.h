@@ -236,7 +236,9 @@ tr_status tr_walk_sweep(const tr_tree* t, double* F_out, double* e_out, uint8_t*
  * serving loop admits requests between launches and splits large ones into
  * Morton ranges, so that small requests are not held up by large ones.
  * trees, first, count: HOST arrays of n >= 1 entries.  Synchronises
- * `stream`.  Errors: TR_EINVAL, TR_ENOMEM, TR_ECUDA, TR_EOVERFLOW. */
+ * `stream`.  Errors: TR_EINVAL, TR_ENOMEM, TR_ECUDA, TR_EOVERFLOW,
+ * TR_EUNSUPPORTED (ray bins of some tree larger than a CTA's shared memory:
+ * then no tree is walked). */
 tr_status tr_walk_sweep_batch(const tr_tree* const* trees, const int64_t* first, const int64_t* count,
                               int32_t n, double* const* F_out, double* const* e_out,
                               uint8_t* const* ion_out, tr_stream stream);

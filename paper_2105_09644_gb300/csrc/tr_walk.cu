@@ -2111,10 +2111,8 @@ tr_status launch_jobs_v(int mode, int out, size_t smem, const WalkArgs* jobs, co
 // limit on a target's bins whichever CTA size is picked.
 constexpr size_t OWN_SMEM_F32 = 19072, OWN_SMEM_F64 = 40512;
 
-// var: some job uses a kernel choice other than W_p / W_f,3 or a boundary
-// other than isolated
-tr_status launch_jobs(int mode, int out, bool var, size_t smem, const WalkArgs* jobs, const int64_t* job_end,
-                      int n_jobs, int64_t total, unsigned int* counter, cudaStream_t st) {
+// The one refusal of a walk: bins that no CTA can hold.
+tr_status check_bins(int mode, int out, size_t smem) {
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     tr_status c = cuda_check(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev),
@@ -2125,6 +2123,15 @@ tr_status launch_jobs(int mode, int out, bool var, size_t smem, const WalkArgs* 
         return set_error(TR_EUNSUPPORTED,
                          "ray bins need %zu + %zu bytes of shared memory per target, more than the %d a CTA can have"
                          " (fewer rays, a shorter L_ray or no e_prev)", smem, own, optin);
+    return TR_OK;
+}
+
+// var: some job uses a kernel choice other than W_p / W_f,3 or a boundary
+// other than isolated
+tr_status launch_jobs(int mode, int out, bool var, size_t smem, const WalkArgs* jobs, const int64_t* job_end,
+                      int n_jobs, int64_t total, unsigned int* counter, cudaStream_t st) {
+    const tr_status c = check_bins(mode, out, smem);
+    if (c != TR_OK) return c;
     return var ? launch_jobs_v<true>(mode, out, smem, jobs, job_end, n_jobs, total, counter, st)
                : launch_jobs_v<false>(mode, out, smem, jobs, job_end, n_jobs, total, counter, st);
 }
@@ -2201,6 +2208,16 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
     // to fill the GPU a few times over joins the next with larger bins.
     struct Item { int tree, per_sm; size_t smem; };
     const int mode = trees[0]->mode;
+    tr_status s = TR_OK;
+    // a batch with a tree that cannot be walked, an idle one too, is refused as
+    // a whole, before anything is launched
+    size_t largest = 0;
+    bool any = false;
+    for (int i = 0; i < n; ++i) {
+        largest = std::max(largest, walk_smem(trees[i]));
+        any = any || count[i] > 0;
+    }
+    if (any && (s = check_bins(mode, OUT_FUSED, largest)) != TR_OK) return s;
     std::vector<Item> items;
     for (int i = 0; i < n; ++i)
         if (count[i] > 0) {
@@ -2216,7 +2233,6 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
     int64_t* he = reinterpret_cast<int64_t*>(host.data() + (size_t)n * sizeof(WalkArgs));
     struct Group { int first, n; size_t smem; int64_t total; bool var; };
     std::vector<Group> groups;
-    tr_status s = TR_OK;
     for (int k = 0; k < (int)items.size(); ++k) {
         const int i = items[k].tree;
         const bool join = k > 0 && (items[k].per_sm == items[k - 1].per_sm ||
@@ -2248,6 +2264,9 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
         if (s == TR_OK)
             s = launch_jobs(mode, OUT_FUSED, g.var, g.smem, jobs + g.first, job_end + g.first, g.n, g.total, counter, st);
     }
+    // an earlier group may be running: it uses the caller's outputs and the
+    // shared job records, which the caller may reuse after an error
+    if (s != TR_OK) cudaStreamSynchronize(st);
     return s;
 }
 
