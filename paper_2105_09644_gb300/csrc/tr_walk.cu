@@ -281,8 +281,9 @@ __device__ __forceinline__ bool bin_nonzero(const double* slot) {
     return (v.x | v.y) != 0u;
 }
 
-// FP32 forms: add v >= 0 (in units of the bin, below 2^62), rounded down to an
-// integer, to a bin.  Integer placement of the significand rather than two
+// FP32 forms: add v >= +0 (in units of the bin, below 2^62; the caller sees to
+// it: the sign bit would be read as part of the exponent, so that -0 would add
+// 2^33 units), rounded down to an integer, to a bin.  Integer placement of the significand rather than two
 // float-to-integer conversions: those share a pipe of 16 lanes per SM and
 // clock (turbulent128, double-FP32 form: 232 -> 226 ms; the unconditional
 // second atomic 226 -> 217 ms).
@@ -303,7 +304,7 @@ __device__ __forceinline__ void bin_add_units(double* slot, float v) {
 template <int MODE>
 __device__ __forceinline__ void bin_atomic_add(double* slot, typename Prec<MODE>::real x, float scale) {
     if constexpr (MODE == 0) atomicAdd(slot, (double)x);
-    else bin_add_units(slot, (float)x * scale);               // exact: scale is a power of two
+    else if ((float)x > 0.f) bin_add_units(slot, (float)x * scale);   // exact: scale is a power of two
 }
 
 template <int MODE>
@@ -1510,6 +1511,10 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
                         radial_setup_exact<MODE>(a, n, exact_d(), s, wcol, gauss);
                     alpha = qv[0];
                     e = a.use_e ? qv[2] : real(0);
+                    if constexpr (MODE != 0) {               // a fixed-point bin takes no addend below +0 (nor -0, NaN)
+                        alpha = alpha > 0.f ? alpha : 0.f;
+                        e = e > 0.f ? e : 0.f;
+                    }
                 }
             }
         }
