@@ -128,6 +128,7 @@ __device__ __forceinline__ float narrow(double a) {
 
 // Comparisons of non-negative doubles: their bit patterns order like them.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }   // of either sign
 __device__ __forceinline__ bool less(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
 
 // W_p of App. A (Eq. A2), outer branch rebuilt from the constraints printed
@@ -1583,7 +1584,7 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
                                      ? radial_w<double>(fabs(radius_at<double>((int)(pk & 0x7fu) + j, a.r_coef, a.r) - d), hpar, VAR ? a.kern_a : 0)
                                      : wc[j * 32];
                 if (positive(ca)) atomicAdd(bins.a + b0 + j, w * ca);
-                if (use_e && positive(ce)) atomicAdd(bins.e + b0 + j, w * ce);
+                if (use_e && nonzero(ce)) atomicAdd(bins.e + b0 + j, w * ce);   // (with its sign: e is the caller's)
             }
         } else {
             // ((W b) cnt) (alpha scale / TW): the scales are powers of two
