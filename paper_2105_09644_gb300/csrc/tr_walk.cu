@@ -1623,15 +1623,19 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
 // a step could overflow it (three full batches of 32 per warp) and at the end.
 template <int NT> constexpr int acc_cap() { return 4 * NT; }
 
-// Opened nodes waiting in a target's ring buffer.  It never holds more than
-// the target's opened nodes (a few hundred at theta = 0.5); overflow is
-// detected and reported, never written past.  While at most FIFO_MAX wait,
-// the oldest are taken first, so that the list fills level by level and a
-// batch of 32 accepted nodes has like numbers of points and rays; beyond
-// that the newest (a depth-first walk, which bounds the buffer: 64 waiting
-// nodes and one step's pushes are what it holds at the same depth).
+// Opened nodes waiting in a target's ring buffer.  While at most FIFO_MAX
+// wait, the oldest are taken first, so that the list fills level by level and
+// a batch of 32 accepted nodes has like numbers of points and rays; beyond
+// that the newest (a depth-first walk, which bounds the buffer).  A step takes
+// no more parents than the room left can hold the children of (7 more than it
+// takes out each), less STACK_RESERVE: where that leaves none, one parent at a
+// time, which needs at most 7 places for each of the levels 2 to 8 below it.
+// So the buffer holds any walk of up to 10 levels, at any opening angle and CTA
+// size (128^3 with e at theta 0.1: 589 places without the bound and 256
+// threads); overflow is still detected and reported, never written past.
 constexpr int STACK_CAP = 512;
 constexpr int FIFO_MAX = 64;
+constexpr int STACK_RESERVE = 7 * (MAX_LEVELS - 1);
 
 // A CTA of NT threads per target.  Walk step: take NT/8 opened nodes from the
 // shared buffer, evaluate their NT children, one per thread; opened children
@@ -1793,7 +1797,7 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
                 spread_list(top == 0 ? nl : nl / NT * NT, img);
                 if (top == 0) break;
             }
-            const int np = min(P, top);
+            const int np = min(min(P, top), max((STACK_CAP - STACK_RESERVE - top) / 7, 1));
             const int pi = tid >> 3, c = tid & 7;
             const bool fifo = top <= FIFO_MAX;
             const uint32_t pe = (pi < np) ? stack[(head + (fifo ? 0 : top - np) + pi) & (STACK_CAP - 1)] : 0u;
