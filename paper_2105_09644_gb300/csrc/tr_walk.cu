@@ -393,11 +393,14 @@ __device__ __forceinline__ double exact_d2(const WalkArgs& a, int64_t nid, float
 // the lane keeps in its column of the warp's NodeBatch, times b; a support
 // of more than MAXW points is evaluated again for each ray instead (`lng`:
 // column entries 0 and 1 then hold d and the kernel's size argument).
-// Kernel values kept per node.  FP32: 8, so that five CTAs fit an SM beside
-// 33 KB of ray bins (N_PIX 48, N_R 43; with 12 only four do: 225 -> 253 ms);
-// a longer support, met by the few nodes with edges of 32 cells and more,
-// costs its evaluation again per ray.  FP64: 12, evaluating again costs more.
-template <int MODE> constexpr int MAXW = MODE == 0 ? 12 : 8;
+// Kernel values kept per node.  FP32: 7, so that a 128-thread CTA takes 9.7 KB
+// beside its ray bins and as many targets fit an SM as should: five at 33 KB of
+// bins (N_PIX 48, N_R 43; with 12 values only four: 225 -> 253 ms), four at 45
+// KB (N_R 59; with 8 only three, by 256 bytes: a 256^3 grid with 100 sources
+// 406 -> 329 ms per 10^6 targets, headline form).  A longer support, met by the
+// few nodes with edges of 32 cells and more, costs its evaluation again per
+// ray.  FP64: 12, evaluating again costs more.
+template <int MODE> constexpr int MAXW = MODE == 0 ? 12 : 7;
 
 template <int MODE>
 struct RadialSpread {
@@ -1667,6 +1670,10 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
     __shared__ __align__(16) WalkArgs s_a;                       // the current job
     __shared__ NodeBatch<MODE> s_nb[NW];
     __shared__ uint32_t s_acc[acc_cap<NT>()];
+    // (228 KB an SM, 1 KB of it the system's per CTA; 48 rays of 59 points, alpha and eps)
+    static_assert(MODE == 0 || NT != 128 ||
+                      sizeof s_nb + sizeof s_acc + sizeof s_a + sizeof s_red + 32 <= 228 * 1024 / 4 - 1024 - 48 * 59 * 16 - STACK_CAP * 4,
+                  "four targets of a 256^3 grid fit an SM");
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const WalkArgs& a = s_a;
     const unsigned lanemask_lt = (1u << lane) - 1u;
@@ -2055,65 +2062,94 @@ tr_status launch_persistent(K kernel, size_t smem, const WalkArgs* jobs, const i
     return cuda_check(cudaGetLastError(), "walk kernel launch");
 }
 
-// Warps that one SM holds of a walk kernel with `smem` bytes of bins and
+// CTAs that one SM holds of a walk kernel with `smem` bytes of bins and
 // buffer (0: it does not fit).
 template <int NT, typename K>
-int resident_warps(K kernel, size_t smem) {
+int resident_ctas(K kernel, size_t smem) {
     int per_sm = 0;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
-    return per_sm * (NT / 32);
+    return per_sm;
 }
 
-// The walk kernel of one form and output, in the CTA size that puts the most
-// warps on an SM, the smaller one of equals: the walk waits on memory and on
-// its barriers, and the ray bins' shared memory sets how many targets an SM
-// holds.  128 threads: five CTAs at 33 KB of bins (N_PIX 48, N_R 43), six
-// when the bins leave room (N_R <= ~30: 64^3 and 32^3 grids 6% faster than
-// with five); 256 and 512 when the bins fill half or most of an SM (N_PIX
-// 192).  At equal warps the smaller CTA waits less at its barriers
-// (turbulent128: 128 x 5 225 ms, 256 x 4 238 ms).  MODE 2 (double-FP32
-// sweep) only differs from MODE 1 in the sweep, so its dump and
-// column-density walks are those of MODE 1 (chosen by launch_jobs).
+// The CTA of a walk: 128 threads with registers for five (K5) or six (K6) on an
+// SM, 256 or 512 threads; and the CTAs that an SM then holds.
+enum CtaKind { K5, K6, K256, K512 };
+struct CtaPick { CtaKind kind = K5; int per_sm = 0; };
+
+// The ray bins' shared memory sets how many targets an SM holds.  Small CTAs
+// hold more of them; large ones bring more warps to each.  A target's sweep by
+// lane pairs keeps 2 N_PIX threads busy whatever the CTA has, so the fused walk
+// takes the CTA with the most threads on an SM that sweep, the most warps
+// among equals (the walk waits on memory and its barriers), the smaller CTA
+// among equals again.  Measured, FP32 + FP64-sweep form, ms:
+//   N_PIX 48, 256^3, 100 sources, 2^20 targets: 4 x 128 329, 2 x 256 515
+//   N_PIX 48, 128^3 with e, 10^3 sources, 2^18: 3 x 128  91, 2 x 256 112
+//   N_PIX 48, 256^3 with e, 100 sources, 2^20:  2 x 128 710, 2 x 256 619
+//   N_PIX 192, 64^3, 10^3 sources, 2^17:        2 x 128  58, 2 x 256  42, 1 x 512 61
+//   N_PIX 192, 64^3 with e, 10^3 sources, 2^16: 1 x 128  69, 1 x 256  46, 1 x 512 39
+// The most warps alone, the rule before, took 2 x 256 in the first two, and the
+// many-source walks of 256^3 grids were slower than with 4 x 128 smaller steps.
+// The dump walk does not sweep: most warps.  MODE 2 (double-FP32 sweep) only
+// differs from MODE 1 in the sweep, so its dump and column-density walks are
+// those of MODE 1 (chosen by launch_jobs).
 template <int MODE, int OUT, bool VAR>
-tr_status launch_sized(size_t smem, const WalkArgs* jobs, const int64_t* job_end, int n_jobs, int64_t total,
+CtaPick pick_cta(size_t smem, int npix) {
+    CtaPick best;
+    int lanes = -1, warps = -1;
+    auto consider = [&](CtaKind kind, int nt, int per_sm) {
+        const int w = per_sm * nt / 32, l = OUT == OUT_FUSED ? per_sm * std::min(nt, 2 * npix) : w;
+        if (l > lanes || (l == lanes && w > warps)) {
+            best = {kind, per_sm};
+            lanes = l;
+            warps = w;
+        }
+    };
+    consider(K5, 128, resident_ctas<128>(k_walk<MODE, OUT, 128, 5, VAR>, smem));
+    if constexpr (OUT == OUT_FUSED && MODE != 0) consider(K6, 128, resident_ctas<128>(k_walk<MODE, OUT, 128, 6, VAR>, smem));
+    consider(K256, 256, resident_ctas<256>(k_walk<MODE, OUT, 256, 2, VAR>, smem));
+    if constexpr (MODE != 0) consider(K512, 512, resident_ctas<512>(k_walk<MODE, OUT, 512, 1, VAR>, smem));
+    return best;
+}
+
+// Ray bins of a launch: the most bytes (with the node buffer) and the most rays
+// of any of its targets.
+struct BinShape { size_t smem; int npix; };
+
+template <int MODE, int OUT, bool VAR>
+tr_status launch_sized(BinShape b, const WalkArgs* jobs, const int64_t* job_end, int n_jobs, int64_t total,
                        unsigned int* counter, cudaStream_t st) {
     auto* const k5 = k_walk<MODE, OUT, 128, 5, VAR>;
-    if constexpr (OUT == OUT_CD) return launch_persistent<128>(k5, smem, jobs, job_end, n_jobs, total, counter, st);
-    auto* const k256 = k_walk<MODE, OUT, 256, 2, VAR>;
-    int best = resident_warps<128>(k5, smem), pick = 0;
-    auto better = [&](int w, int k) { if (w > best) { best = w; pick = k; } };
-    if constexpr (OUT == OUT_FUSED && MODE != 0) better(resident_warps<128>(k_walk<MODE, OUT, 128, 6, VAR>, smem), 1);
-    better(resident_warps<256>(k256, smem), 2);
-    if constexpr (MODE != 0) better(resident_warps<512>(k_walk<MODE, OUT, 512, 1, VAR>, smem), 3);
+    if constexpr (OUT == OUT_CD) return launch_persistent<128>(k5, b.smem, jobs, job_end, n_jobs, total, counter, st);
+    const CtaKind kind = pick_cta<MODE, OUT, VAR>(b.smem, b.npix).kind;
     if constexpr (OUT == OUT_FUSED && MODE != 0)
-        if (pick == 1) return launch_persistent<128>(k_walk<MODE, OUT, 128, 6, VAR>, smem, jobs, job_end, n_jobs, total, counter, st);
+        if (kind == K6) return launch_persistent<128>(k_walk<MODE, OUT, 128, 6, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
     if constexpr (MODE != 0)
-        if (pick == 3) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR>, smem, jobs, job_end, n_jobs, total, counter, st);
-    if (pick == 2) return launch_persistent<256>(k256, smem, jobs, job_end, n_jobs, total, counter, st);
-    return launch_persistent<128>(k5, smem, jobs, job_end, n_jobs, total, counter, st);
+        if (kind == K512) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
+    if (kind == K256) return launch_persistent<256>(k_walk<MODE, OUT, 256, 2, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
+    return launch_persistent<128>(k5, b.smem, jobs, job_end, n_jobs, total, counter, st);
 }
 
 template <int MODE, bool VAR>
-tr_status launch_mode(int out, size_t smem, const WalkArgs* jobs, const int64_t* job_end, int n_jobs, int64_t total,
+tr_status launch_mode(int out, BinShape b, const WalkArgs* jobs, const int64_t* job_end, int n_jobs, int64_t total,
                       unsigned int* counter, cudaStream_t st) {
     if constexpr (MODE != 2) {
-        if (out == OUT_CD) return launch_sized<MODE, OUT_CD, VAR>(smem, jobs, job_end, n_jobs, total, counter, st);
-        if (out == OUT_DUMP) return launch_sized<MODE, OUT_DUMP, VAR>(smem, jobs, job_end, n_jobs, total, counter, st);
+        if (out == OUT_CD) return launch_sized<MODE, OUT_CD, VAR>(b, jobs, job_end, n_jobs, total, counter, st);
+        if (out == OUT_DUMP) return launch_sized<MODE, OUT_DUMP, VAR>(b, jobs, job_end, n_jobs, total, counter, st);
     }
-    return launch_sized<MODE, OUT_FUSED, VAR>(smem, jobs, job_end, n_jobs, total, counter, st);
+    return launch_sized<MODE, OUT_FUSED, VAR>(b, jobs, job_end, n_jobs, total, counter, st);
 }
 
 template <bool VAR>
-tr_status launch_jobs_v(int mode, int out, size_t smem, const WalkArgs* jobs, const int64_t* job_end,
+tr_status launch_jobs_v(int mode, int out, BinShape b, const WalkArgs* jobs, const int64_t* job_end,
                         int n_jobs, int64_t total, unsigned int* counter, cudaStream_t st) {
-    if (mode == 0) return launch_mode<0, VAR>(out, smem, jobs, job_end, n_jobs, total, counter, st);
+    if (mode == 0) return launch_mode<0, VAR>(out, b, jobs, job_end, n_jobs, total, counter, st);
     if (mode == 1 || out != OUT_FUSED)
-        return launch_mode<1, VAR>(out, smem, jobs, job_end, n_jobs, total, counter, st);
-    return launch_mode<2, VAR>(out, smem, jobs, job_end, n_jobs, total, counter, st);
+        return launch_mode<1, VAR>(out, b, jobs, job_end, n_jobs, total, counter, st);
+    return launch_mode<2, VAR>(out, b, jobs, job_end, n_jobs, total, counter, st);
 }
 
 // Shared memory of a CTA that is not for ray bins and the node buffer: what
@@ -2138,31 +2174,18 @@ tr_status check_bins(int mode, int out, size_t smem) {
 
 // var: some job uses a kernel choice other than W_p / W_f,3 or a boundary
 // other than isolated
-tr_status launch_jobs(int mode, int out, bool var, size_t smem, const WalkArgs* jobs, const int64_t* job_end,
+tr_status launch_jobs(int mode, int out, bool var, BinShape b, const WalkArgs* jobs, const int64_t* job_end,
                       int n_jobs, int64_t total, unsigned int* counter, cudaStream_t st) {
-    const tr_status c = check_bins(mode, out, smem);
+    const tr_status c = check_bins(mode, out, b.smem);
     if (c != TR_OK) return c;
-    return var ? launch_jobs_v<true>(mode, out, smem, jobs, job_end, n_jobs, total, counter, st)
-               : launch_jobs_v<false>(mode, out, smem, jobs, job_end, n_jobs, total, counter, st);
+    return var ? launch_jobs_v<true>(mode, out, b, jobs, job_end, n_jobs, total, counter, st)
+               : launch_jobs_v<false>(mode, out, b, jobs, job_end, n_jobs, total, counter, st);
 }
 
 // Targets that an SM holds at once in the fused walk of a form.
-template <int MODE>
-int targets_per_sm_m(size_t smem) {
-    constexpr int F = OUT_FUSED;
-    const int w128 = resident_warps<128>(k_walk<MODE, F, 128, 5, false>, smem), w256 = resident_warps<256>(k_walk<MODE, F, 256, 2, false>, smem);
-    int best = w128, per = w128 / 4;
-    if constexpr (MODE != 0) {
-        const int w6 = resident_warps<128>(k_walk<MODE, F, 128, 6, false>, smem);
-        if (w6 > best) { best = w6; per = w6 / 4; }
-    }
-    if (w256 > best) { best = w256; per = w256 / 8; }
-    if constexpr (MODE != 0)
-        if (resident_warps<512>(k_walk<MODE, F, 512, 1, false>, smem) > best) per = 1;
-    return per;
-}
-int targets_per_sm(int mode, size_t smem) {
-    return mode == 0 ? targets_per_sm_m<0>(smem) : (mode == 1 ? targets_per_sm_m<1>(smem) : targets_per_sm_m<2>(smem));
+int targets_per_sm(int mode, BinShape b) {
+    return (mode == 0 ? pick_cta<0, OUT_FUSED, false>(b.smem, b.npix)
+            : mode == 1 ? pick_cta<1, OUT_FUSED, false>(b.smem, b.npix) : pick_cta<2, OUT_FUSED, false>(b.smem, b.npix)).per_sm;
 }
 constexpr int BATCH_WAVES = 4;              // targets per resident target below which a batch's group is too small
 
@@ -2188,8 +2211,8 @@ tr_status walk_run(const tr_tree* t, const int64_t* targets, int64_t n_targets, 
     const int64_t* job_end = nullptr;
     const tr_status s = job_start(a, t, n_targets, &jobs, &job_end, st);
     if (s != TR_OK || n_targets <= 0) return s;
-    return launch_jobs(t->mode, dump ? OUT_DUMP : OUT_FUSED, uses_variants(t), walk_smem(t), jobs, job_end, 1, n_targets,
-                       t->counter, st);
+    return launch_jobs(t->mode, dump ? OUT_DUMP : OUT_FUSED, uses_variants(t),
+                       {walk_smem(t), t->npix}, jobs, job_end, 1, n_targets, t->counter, st);
 }
 
 tr_status cd_run(const tr_tree* t, const int64_t* targets, int64_t n_targets, double* out, cudaStream_t st) {
@@ -2205,7 +2228,7 @@ tr_status cd_run(const tr_tree* t, const int64_t* targets, int64_t n_targets, do
     const tr_status s = job_start(a, t, n_targets, &jobs, &job_end, st);
     if (s != TR_OK || n_targets <= 0) return s;
     const size_t smem = (size_t)t->npix * 8 + (size_t)STACK_CAP * 4;
-    return launch_jobs(t->mode, OUT_CD, uses_variants(t), smem, jobs, job_end, 1, n_targets, t->counter, st);
+    return launch_jobs(t->mode, OUT_CD, uses_variants(t), {smem, t->npix}, jobs, job_end, 1, n_targets, t->counter, st);
 }
 
 tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, const int64_t* count, int n,
@@ -2232,7 +2255,7 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
     for (int i = 0; i < n; ++i)
         if (count[i] > 0) {
             const size_t m = walk_smem(trees[i]);
-            items.push_back({i, targets_per_sm(mode, m), m});
+            items.push_back({i, targets_per_sm(mode, {m, trees[i]->npix}), m});
         }
     std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.per_sm > y.per_sm; });
     int dev = 0, sms = 0;
@@ -2241,13 +2264,13 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
     std::vector<unsigned char> host(walk_job_bytes(n));
     WalkArgs* hj = reinterpret_cast<WalkArgs*>(host.data());
     int64_t* he = reinterpret_cast<int64_t*>(host.data() + (size_t)n * sizeof(WalkArgs));
-    struct Group { int first, n; size_t smem; int64_t total; bool var; };
+    struct Group { int first, n; BinShape b; int64_t total; bool var; };
     std::vector<Group> groups;
     for (int k = 0; k < (int)items.size(); ++k) {
         const int i = items[k].tree;
         const bool join = k > 0 && (items[k].per_sm == items[k - 1].per_sm ||
                                     groups.back().total < (int64_t)sms * items[k - 1].per_sm * BATCH_WAVES);
-        if (!join) groups.push_back({k, 0, 0, 0, false});
+        if (!join) groups.push_back({k, 0, {0, 0}, 0, false});
         Group& g = groups.back();
         WalkArgs a = make_args(trees[i]);
         a.targets = nullptr;
@@ -2258,7 +2281,7 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
         ++g.n;
         g.total += count[i];
         he[k] = g.total;
-        g.smem = std::max(g.smem, items[k].smem);
+        g.b = {std::max(g.b.smem, items[k].smem), std::max(g.b.npix, trees[i]->npix)};
         g.var = g.var || uses_variants(trees[i]);
     }
     for (int i = 0; i < n; ++i) {
@@ -2272,7 +2295,7 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
     for (const Group& g : groups) {
         if (s == TR_OK) s = cuda_check(cudaMemsetAsync(counter, 0, sizeof(unsigned int), st), "counter reset");
         if (s == TR_OK)
-            s = launch_jobs(mode, OUT_FUSED, g.var, g.smem, jobs + g.first, job_end + g.first, g.n, g.total, counter, st);
+            s = launch_jobs(mode, OUT_FUSED, g.var, g.b, jobs + g.first, job_end + g.first, g.n, g.total, counter, st);
     }
     // an earlier group may be running: it uses the caller's outputs and the
     // shared job records, which the caller may reuse after an error
