@@ -128,7 +128,7 @@ __device__ __forceinline__ float narrow(double a) {
 
 // Comparisons of non-negative doubles: their bit patterns order like them.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
-__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }   // of either sign
+__device__ __forceinline__ bool nonzero(double x) { return (__double2hiint(x) | __double2loint(x)) != 0; }   // (or -0)
 __device__ __forceinline__ bool less(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
 
 // W_p of App. A (Eq. A2), outer branch rebuilt from the constraints printed
@@ -1804,7 +1804,8 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
                 spread_list(top == 0 ? nl : nl / NT * NT, img);
                 if (top == 0) break;
             }
-            const int np = min(min(P, top), max((STACK_CAP - STACK_RESERVE - top) / 7, 1));
+            int np = min(P, top);
+            if (top > STACK_CAP - STACK_RESERVE - 7 * P) np = max(min(np, (STACK_CAP - STACK_RESERVE - top) / 7), 1);
             const int pi = tid >> 3, c = tid & 7;
             const bool fifo = top <= FIFO_MAX;
             const uint32_t pe = (pi < np) ? stack[(head + (fifo ? 0 : top - np) + pi) & (STACK_CAP - 1)] : 0u;
