@@ -994,6 +994,9 @@ __device__ __forceinline__ double sweep_ray_group(const WalkArgs& a, const doubl
 constexpr int MAX_NPIX = 12 * 8 * 8;                  // N_side <= 8
 constexpr int GROUP_MAX = 32;                         // rays with more points go to lane pairs
 constexpr int GROUP_MEAN_MAX = 14;                    // lane groups while a lit ray has at most this many points on average
+// FP64 sweeps: lane groups while a target's fill at most this many lanes (see
+// sweep_rays)
+__device__ __forceinline__ int group_lanes_max(int npix) { return max(128, 4 * npix / 3); }
 constexpr int N_CLS = 7;                              // classes of rays with emitting points
 struct RayScratch {
     uint32_t* cls;
@@ -1260,19 +1263,22 @@ __device__ __forceinline__ double sweep_groups(const WalkArgs& a, const double* 
 // rotates which warps take the work from target to target.
 // FP64 sweeps (FP64 form and FP32 + FP64-sweep form): rays with a lone source
 // by a warp each (lone_ray).  Of the others, while their points fill at most
-// one lane group position per thread of the CTA, all warps ready the rays
+// group_lanes_max lanes, all warps ready the rays
 // (prepare_ray) and sweep them a lane per point (sweep_group64; more than
 // GROUP_MAX points: lane pairs): the fewest FP64 instructions in a row, and the
 // target's time is that chain.  Beyond that the FP64 units are what is short,
 // and lane pairs, 16 rays of like load to a warp, take fewest in all (a lane
 // for a point that the sweep has not reached costs as much as a busy one).
-// turbulent128 278 -> 236 ms with this rule, 275 with pairs only, 251 with half
-// the threads as the line; AMR 64^3 at N_PIX 192 35 ms with groups only, 24
-// with the rule.  Coefficients computed within the chain where lane pairs
+// The line lies at 128 lanes for up to 96 rays (turbulent128 278 -> 236 ms
+// with it, 275 with pairs only, 251 with 64 lanes) and at 4/3 of a lane per ray
+// beyond (N_PIX 192, 64^3, 10 sources: 23.1 ms with 256 lanes, 23.9 with 128; AMR 64^3
+// 24 ms, 35 with groups only).  Coefficients computed within the chain where lane pairs
 // sweep: 505 -> 492 ms for 10^4 sources at 128^3 (its FP64 units are busy).
 // Double-FP32 sweep: lane groups up to GROUP_MEAN_MAX points per lit ray on
 // average (sweep_groups), lane pairs beyond (sweep_ray_group).  The choices
-// depend only on the bins.  `scratch` holds sweep_scratch_bytes bytes of
+// depend only on the bins and N_PIX, so a target's rays are swept alike in a CTA
+// of any size, alone, in a batch or from stored bins; only the order of the sum
+// over the rays follows the CTA.  `scratch` holds sweep_scratch_bytes bytes of
 // shared memory; all threads call.
 template <int MODE, int NT>
 __device__ __forceinline__ double sweep_rays(const WalkArgs& a, double* bins_a, double* bins_eps, double* bins_e,
@@ -1287,7 +1293,7 @@ __device__ __forceinline__ double sweep_rays(const WalkArgs& a, double* bins_a, 
     if constexpr (MODE != 2) {
         const int wid = ((tid >> 5) + turn) & (NW - 1);       // its place in the sum too (block_sum)
         const int n_lone = use_e ? 0 : rk.none, T = rk.lanes - n_lone, n_more = rk.nz - n_lone;
-        const bool groups = T <= NT, ready = groups || use_e;
+        const bool groups = T <= group_lanes_max(a.npix), ready = groups || use_e;
         for (int r = (ready ? 0 : n_more) + wid; r < rk.nz; r += NW) {
             const int k = rs.order[r];
             ray_mask(bins_eps, rs, nr, k, m0, m1);
