@@ -400,7 +400,8 @@ __device__ __forceinline__ double exact_d2(const WalkArgs& a, int64_t nid, float
 // 406 -> 329 ms per 10^6 targets, headline form).  A longer support, met by the
 // few nodes with edges of 32 cells and more, costs its evaluation again per
 // ray.  FP64: 12, evaluating again costs more.
-template <int MODE> constexpr int MAXW = MODE == 0 ? 12 : 7;
+// SLIM: the 512-thread CTA beside bins of 190 to 199 KB (see pick_cta).
+template <int MODE, bool SLIM = false> constexpr int MAXW = MODE == 0 ? 12 : (SLIM ? 6 : 7);
 
 template <int MODE>
 struct RadialSpread {
@@ -413,10 +414,10 @@ struct RadialSpread {
 // memory: kernel values in a column per set-up lane (conflict-free for lanes
 // that read different nodes at the same point), the rest by the node's rank
 // among the nodes with work.
-template <int MODE>
+template <int MODE, int W>
 struct __align__(16) NodeBatch {
     using real = typename Prec<MODE>::real;
-    real w[MAXW<MODE>][32];
+    real w[W][32];
     uint2 key[32];                          // {first table entry less first (node, ray) pair, points packed}
     real a[32], b[32];                      // alpha, weight factor (FP64 form: alpha x b / TW, -)
     real e[32];                             // e (FP64 form: e x b / TW)
@@ -440,7 +441,7 @@ __device__ __forceinline__ T radius_at(int i, T coef, const double* tab) {
 // not, or a support that is empty or holds only points within rounding of
 // its edge (the normalisation then jumps between one point and the linear
 // split) -- is not settled in FP32; radial_setup_exact then takes it in FP64.
-template <int MODE>
+template <int MODE, int W>
 __device__ __forceinline__ bool radial_setup(const WalkArgs& a, RadialSpread<MODE>& n, float d, int s, float* wcol, int gauss,
                                              float dtol) {
     using real = float;
@@ -477,7 +478,7 @@ __device__ __forceinline__ bool radial_setup(const WalkArgs& a, RadialSpread<MOD
         if (w > real(0)) {                  // the support is one run of points
             S += w;
             last = i;
-            if (cnt < MAXW<MODE>) *col = w;
+            if (cnt < W) *col = w;
             col += 32;
             ++cnt;
         }
@@ -492,7 +493,7 @@ __device__ __forceinline__ bool radial_setup(const WalkArgs& a, RadialSpread<MOD
     }
     if (cnt > 0) {
         n.lo = last - cnt + 1; n.npts = cnt; n.b = real(1) / S;
-        if (cnt > MAXW<MODE>) { n.lng = true; wcol[0] = d; wcol[32] = hpar; }
+        if (cnt > W) { n.lng = true; wcol[0] = d; wcol[32] = hpar; }
         return false;
     }
     int i = min(max((int)floorf((float)a.eta * sqrtf(2.f * (float)d)), 0), nr - 2);   // a guess, corrected below
@@ -1453,8 +1454,8 @@ struct Bins {
 // lanes full, which a thread that evaluates a node and then spreads it
 // cannot: at theta = 0.5 three quarters of the evaluated nodes are accepted,
 // and a node has 1 to 20 rays and 1 to 10 points.
-template <int MODE, int OUT, bool VAR>
-__device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>& nb, uint32_t entry, bool have, int img,
+template <int MODE, int OUT, bool VAR, int W>
+__device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE, W>& nb, uint32_t entry, bool have, int img,
                                              const Target<MODE>& t, const Bins& bins, const Scales& sc, float kap,
                                              WalkCounters& cnt) {
     using real = typename Prec<MODE>::real;
@@ -1517,7 +1518,7 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
                     const int gauss = VAR ? a.kern_a : 0;
                     real* const wcol = &nb.w[0][lane];
                     if constexpr (MODE == 0) radial_setup64(a, n, d, s, wcol, gauss);
-                    else if (radial_setup<MODE>(a, n, d, s, wcol, gauss, dtol))
+                    else if (radial_setup<MODE, W>(a, n, d, s, wcol, gauss, dtol))
                         radial_setup_exact<MODE>(a, n, exact_d(), s, wcol, gauss);
                     alpha = qv[0];
                     e = a.use_e ? qv[2] : real(0);
@@ -1630,7 +1631,8 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE>&
 
 // The list of accepted nodes waiting to be spread: 4 NT entries, spread when
 // a step could overflow it (three full batches of 32 per warp) and at the end.
-template <int NT> constexpr int acc_cap() { return 4 * NT; }
+// SLIM: 2 NT, spread one batch per warp at a time.
+template <int NT, bool SLIM> constexpr int acc_cap() { return (SLIM ? 2 : 4) * NT; }
 
 // Opened nodes waiting in a target's ring buffer.  While at most FIFO_MAX
 // wait, the oldest are taken first, so that the list fills level by level and
@@ -1657,7 +1659,7 @@ constexpr int STACK_RESERVE = 7 * (MAX_LEVELS - 1);
 // before, left a third of the lanes idle and took turbulent128 from 217 to
 // 328 ms in the double-FP32 form (99 k to 62 k warp instructions per target
 // in the headline form).
-template <int MODE, int OUT, int NT, bool VAR>
+template <int MODE, int OUT, int NT, bool VAR, bool SLIM>
 __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, const int64_t* __restrict__ job_end,
                                           int n_jobs, unsigned int* counter) {
     using real = typename Prec<MODE>::real;
@@ -1674,8 +1676,8 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
     __shared__ int s_j;
     __shared__ int s_nacc;
     __shared__ __align__(16) WalkArgs s_a;                       // the current job
-    __shared__ NodeBatch<MODE> s_nb[NW];
-    __shared__ uint32_t s_acc[acc_cap<NT>()];
+    __shared__ NodeBatch<MODE, MAXW<MODE, SLIM>> s_nb[NW];
+    __shared__ uint32_t s_acc[acc_cap<NT, SLIM>()];
     // (228 KB an SM, 1 KB of it the system's per CTA; 48 rays of 59 points, alpha and eps)
     static_assert(MODE == 0 || NT != 128 ||
                       sizeof s_nb + sizeof s_acc + sizeof s_a + sizeof s_red + 32 <= 228 * 1024 / 4 - 1024 - 48 * 59 * 16 - STACK_CAP * 4,
@@ -1806,7 +1808,7 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
             __syncthreads();                                     // the image's root visible, the list read
         }
         for (;;) {
-            if (top == 0 || nl + NT > acc_cap<NT>()) {           // the walk's end, or a full list: full batches
+            if (top == 0 || nl + NT > acc_cap<NT, SLIM>()) {           // the walk's end, or a full list: full batches
                 spread_list(top == 0 ? nl : nl / NT * NT, img);
                 if (top == 0) break;
             }
@@ -1950,10 +1952,10 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
 }
 
 // CTAS: the CTAs per SM that the registers have to allow.
-template <int MODE, int OUT, int NT, int CTAS, bool VAR>
+template <int MODE, int OUT, int NT, int CTAS, bool VAR, bool SLIM = false>
 __global__ void __launch_bounds__(NT, CTAS) k_walk(const WalkArgs* __restrict__ jobs, const int64_t* __restrict__ job_end,
                                                   int n_jobs, unsigned int* counter) {
-    walk_body<MODE, OUT, NT, VAR>(jobs, job_end, n_jobs, counter);
+    walk_body<MODE, OUT, NT, VAR, SLIM>(jobs, job_end, n_jobs, counter);
 }
 
 // Unfused sweep over bins stored by the dump walk: one CTA per target.
@@ -2083,8 +2085,9 @@ int resident_ctas(K kernel, size_t smem) {
 }
 
 // The CTA of a walk: 128 threads with registers for five (K5) or six (K6) on an
-// SM, 256 or 512 threads; and the CTAs that an SM then holds.
-enum CtaKind { K5, K6, K256, K512 };
+// SM, 256 or 512 threads; 512 with less memory of its own; and the CTAs that an
+// SM then holds.
+enum CtaKind { K5, K6, K256, K512, K512_SLIM };
 struct CtaPick { CtaKind kind = K5; int per_sm = 0; };
 
 // The ray bins' shared memory sets how many targets an SM holds.  Small CTAs
@@ -2100,7 +2103,10 @@ struct CtaPick { CtaKind kind = K5; int per_sm = 0; };
 //   N_PIX 192, 64^3 with e, 10^3 sources, 2^16: 1 x 128  69, 1 x 256  46, 1 x 512 39
 // The most warps alone, the rule before, took 2 x 256 in the first two, and the
 // many-source walks of 256^3 grids were slower than with 4 x 128 smaller steps.
-// The dump walk does not sweep: most warps.  MODE 2 (double-FP32 sweep) only
+// The slim 512-thread CTA (31 KB of its own instead of 37) is for bins that
+// leave the other no room, as 128^3 grids with e at N_PIX 192 do (double-FP32
+// form, 10^3 sources, 2^16 targets: 256 threads 73 ms, slim 50 ms); where both
+// fit it is 2 to 10% slower.  The dump walk does not sweep: most warps.  MODE 2 (double-FP32 sweep) only
 // differs from MODE 1 in the sweep, so its dump and column-density walks are
 // those of MODE 1 (chosen by launch_jobs).
 template <int MODE, int OUT, bool VAR>
@@ -2119,6 +2125,8 @@ CtaPick pick_cta(size_t smem, int npix) {
     if constexpr (OUT == OUT_FUSED && MODE != 0) consider(K6, 128, resident_ctas<128>(k_walk<MODE, OUT, 128, 6, VAR>, smem));
     consider(K256, 256, resident_ctas<256>(k_walk<MODE, OUT, 256, 2, VAR>, smem));
     if constexpr (MODE != 0) consider(K512, 512, resident_ctas<512>(k_walk<MODE, OUT, 512, 1, VAR>, smem));
+    if constexpr (OUT == OUT_FUSED && MODE != 0)
+        consider(K512_SLIM, 512, resident_ctas<512>(k_walk<MODE, OUT, 512, 1, VAR, true>, smem));
     return best;
 }
 
@@ -2134,6 +2142,8 @@ tr_status launch_sized(BinShape b, const WalkArgs* jobs, const int64_t* job_end,
     const CtaKind kind = pick_cta<MODE, OUT, VAR>(b.smem, b.npix).kind;
     if constexpr (OUT == OUT_FUSED && MODE != 0)
         if (kind == K6) return launch_persistent<128>(k_walk<MODE, OUT, 128, 6, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
+    if constexpr (OUT == OUT_FUSED && MODE != 0)
+        if (kind == K512_SLIM) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR, true>, b.smem, jobs, job_end, n_jobs, total, counter, st);
     if constexpr (MODE != 0)
         if (kind == K512) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
     if (kind == K256) return launch_persistent<256>(k_walk<MODE, OUT, 256, 2, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
