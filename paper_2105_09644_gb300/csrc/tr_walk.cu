@@ -2106,9 +2106,9 @@ struct CtaPick { CtaKind kind = K5; int per_sm = 0; };
 // The slim 512-thread CTA (31 KB of its own instead of 37) is for bins that
 // leave the other no room, as 128^3 grids with e at N_PIX 192 do (double-FP32
 // form, 10^3 sources, 2^16 targets: 256 threads 73 ms, slim 50 ms); where both
-// fit it is 2 to 10% slower.  The dump walk does not sweep: most warps.  MODE 2 (double-FP32 sweep) only
-// differs from MODE 1 in the sweep, so its dump and column-density walks are
-// those of MODE 1 (chosen by launch_jobs).
+// fit it is 2 to 10% slower.  The dump walk does not sweep: most warps.  MODE 2
+// (double-FP32 sweep) only differs from MODE 1 in the sweep, so its dump and
+// column-density walks are those of MODE 1 (chosen by launch_jobs).
 template <int MODE, int OUT, bool VAR>
 CtaPick pick_cta(size_t smem, int npix) {
     CtaPick best;
@@ -2123,10 +2123,16 @@ CtaPick pick_cta(size_t smem, int npix) {
     };
     consider(K5, 128, resident_ctas<128>(k_walk<MODE, OUT, 128, 5, VAR>, smem));
     if constexpr (OUT == OUT_FUSED && MODE != 0) consider(K6, 128, resident_ctas<128>(k_walk<MODE, OUT, 128, 6, VAR>, smem));
-    consider(K256, 256, resident_ctas<256>(k_walk<MODE, OUT, 256, 2, VAR>, smem));
-    if constexpr (MODE != 0) consider(K512, 512, resident_ctas<512>(k_walk<MODE, OUT, 512, 1, VAR>, smem));
-    if constexpr (OUT == OUT_FUSED && MODE != 0)
-        consider(K512_SLIM, 512, resident_ctas<512>(k_walk<MODE, OUT, 512, 1, VAR, true>, smem));
+    // (registers allow two CTAs of 256 threads and one of 512: not asked where that cannot win)
+    auto worth = [&](int nt, int per_sm) { return OUT != OUT_FUSED || per_sm * std::min(nt, 2 * npix) >= lanes; };
+    if (worth(256, 2)) consider(K256, 256, resident_ctas<256>(k_walk<MODE, OUT, 256, 2, VAR>, smem));
+    if constexpr (MODE != 0)
+        if (worth(512, 1)) {
+            const int n = resident_ctas<512>(k_walk<MODE, OUT, 512, 1, VAR>, smem);
+            consider(K512, 512, n);
+            if constexpr (OUT == OUT_FUSED)
+                if (n == 0) consider(K512_SLIM, 512, resident_ctas<512>(k_walk<MODE, OUT, 512, 1, VAR, true>, smem));
+        }
     return best;
 }
 
