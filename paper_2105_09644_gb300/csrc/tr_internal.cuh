@@ -81,15 +81,39 @@ __host__ __device__ inline uint32_t morton3(uint32_t x, uint32_t y, uint32_t z) 
 }
 
 #ifdef __CUDACC__
-// A float >= 0 as a double, by integer operations (subnormals give 0): GB300's
-// FP64 units also do the conversions, at 64 cycles per warp instruction.
-__device__ __forceinline__ double widen(float f) {
+// A float as a double, by integer operations: GB300's FP64 units also do the
+// conversions, at 64 cycles per warp instruction.
+// +0 or a normal number > 0:
+__device__ __forceinline__ double widen_normal(float f) {
     const uint32_t b = __float_as_uint(f);
-    return b < 0x00800000u ? 0.0 : __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+    return b == 0u ? 0.0 : __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
+// The same times 2^k, base = 0x38000000 + (k << 20), a result in the normal range:
+__device__ __forceinline__ double widen_scaled(float f, int base) {
+    const uint32_t b = __float_as_uint(f);
+    return __hiloint2double(b ? (int)(b >> 3) + base : 0, (int)(b << 29));
+}
+// Of either sign; subnormals give 0.  Not for infinities and NaN.
 __device__ __forceinline__ double widen_signed(float f) {
-    const double d = widen(fabsf(f));
-    return __hiloint2double(__double2hiint(d) | (int)(__float_as_uint(f) & 0x80000000u), __double2loint(d));
+    const uint32_t b = __float_as_uint(f), m = b & 0x7fffffffu;
+    return m < 0x00800000u ? __hiloint2double((int)(b - m), 0)
+                           : __hiloint2double((int)(((m >> 3) + 0x38000000u) | (b - m)), (int)(b << 29));
+}
+// n floats, any: by integer operations where all are zero or normal, which one
+// test of their largest and smallest patterns decides.
+template <int n>
+__device__ __forceinline__ void widen_all(const float (&f)[n], double (&d)[n]) {
+    uint32_t hi = 0u, lo = 0xffffffffu;
+    for (int k = 0; k < n; ++k) {
+        const uint32_t m = __float_as_uint(f[k]) & 0x7fffffffu;
+        hi = max(hi, m);
+        lo = min(lo, m - 1u);                                 // (zero last)
+    }
+    if (hi < 0x7f800000u && lo >= 0x007fffffu) {
+        for (int k = 0; k < n; ++k) d[k] = widen_signed(f[k]);
+    } else {
+        for (int k = 0; k < n; ++k) asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d[k]) : "f"(f[k]));   // (stays in its branch)
+    }
 }
 #endif
 

@@ -82,7 +82,7 @@ __device__ __forceinline__ int padded(int i) { return i + (i >> 3); }
 // residual r decides: |r| / m below half an ulp of p.  Two FP64 instructions
 // instead of a division.
 __device__ __forceinline__ double cell_centre(double m, float pf, double& mp) {
-    const double p = widen(pf);
+    const double p = widen_normal(pf);
     mp = __dmul_rn(m, p);
     if (!(__double2hiint(m) > 0x10000000)) return m > 0.0 ? __ddiv_rn(mp, m) : p;   // tiny or no mass
     const double r = fabs(fma(-m, p, mp));
@@ -155,8 +155,9 @@ __global__ void __launch_bounds__(BUILD_NT, 3) k_build(BuildArgs a) {
                 f32[B_ALPHA][k] = q.alpha; f32[B_EPS][k] = q.eps; f32[B_E][k] = q.e; f32[B_MION][k] = q.mion;
                 const float px = (float)ix + 0.5f, py = (float)iy + 0.5f, pz = (float)iz + 0.5f;
                 auto differs = [](double u, double v) { return __double_as_longlong(u) != __double_as_longlong(v); };
-                if (differs(nd.cmx, widen(px)) || differs(nd.cmy, widen(py)) || differs(nd.cmz, widen(pz))) {
-                    const double ex = fabs(widen(px) - nd.cmx), ey = fabs(widen(py) - nd.cmy), ez = fabs(widen(pz) - nd.cmz);
+                if (differs(nd.cmx, widen_normal(px)) || differs(nd.cmy, widen_normal(py)) || differs(nd.cmz, widen_normal(pz))) {
+                    const double ex = fabs(widen_normal(px) - nd.cmx), ey = fabs(widen_normal(py) - nd.cmy),
+                                 ez = fabs(widen_normal(pz) - nd.cmz);
                     kap = __double2float_ru(fmax(ex, fmax(ey, ez)));
                 }
             }
@@ -219,14 +220,14 @@ __global__ void __launch_bounds__(BUILD_NT, 3) k_build(BuildArgs a) {
                 const int x = f - B_X;
                 const float g = ((float)compact3(m >> x) + 0.5f) * s;   // the geometric centre, exact
                 const double m64 = f64[B_M][k];
-                const double cm = m64 > 0.0 ? __ddiv_rn(sum, m64) : widen(g);
+                const double cm = m64 > 0.0 ? __ddiv_rn(sum, m64) : widen_normal(g);
                 r64[x] = cm;
                 if (start) a.s64[3 * id + x] = sum;
                 if (F32) {
                     const float mf = f32[B_M][k], o = mf > 0.f ? sum32 / mf : 0.f;
                     r32[x] = o;
                     if (start) a.s32[3 * id + x] = sum32;
-                    const double ex = fabs(widen(g) + widen_signed(o) - cm) * widen(1.f / s);   // (s a power of two)
+                    const double ex = fabs(widen_normal(g) + widen_signed(o) - cm) * widen_normal(1.f / s);   // (s a power of two)
                     kap = fmaxf(kap, __double2float_ru(ex));
                 }
             } else {
@@ -456,11 +457,9 @@ __global__ void k_export(const void* nodes_v, int64_t n, double* out, double U, 
         const int l = node_level(i);
         const uint32_t m = (uint32_t)(i - level_offset(l));
         const float s = (float)(N >> l);
-        v[0] = widen(q.m);
-        v[1] = absent ? 0.0 : widen(((float)compact3(m) + 0.5f) * s) + widen_signed(q.ox);
-        v[2] = absent ? 0.0 : widen(((float)compact3(m >> 1) + 0.5f) * s) + widen_signed(q.oy);
-        v[3] = absent ? 0.0 : widen(((float)compact3(m >> 2) + 0.5f) * s) + widen_signed(q.oz);
-        v[4] = widen(q.alpha); v[5] = widen(q.eps); v[6] = widen(q.e); v[7] = widen(fabsf(q.mion));
+        const float f[8] = {q.m, q.ox, q.oy, q.oz, q.alpha, q.eps, q.e, fabsf(q.mion)};
+        widen_all(f, v);
+        for (int x = 0; x < 3; ++x) v[1 + x] = absent ? 0.0 : widen_normal(((float)compact3(m >> x) + 0.5f) * s) + v[1 + x];
     }
     v[4] *= U; v[5] *= U; v[6] *= Eu;
     if ((reinterpret_cast<uintptr_t>(out) & 15) == 0) {        // the caller's array need only be aligned to doubles

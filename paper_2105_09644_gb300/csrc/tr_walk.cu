@@ -537,7 +537,7 @@ __device__ __forceinline__ void radial_setup64(const WalkArgs& a, RadialSpread<0
     }
     // s is a power of two: 1 / h from its exponent
     const float hf = (float)s, inv_hf = __uint_as_float((254u << 23) - __float_as_uint(hf));
-    const double h = widen(hf), inv_h = widen(inv_hf), hpar = gauss ? h : inv_h;
+    const double h = widen_normal(hf), inv_h = widen_normal(inv_hf), hpar = gauss ? h : inv_h;
     const float df = narrow(d), reach = 0.8661f * hf, dlo = df > reach ? df - reach : 0.f;
     const float el = 2.f * dlo, eh = 2.f * (df + reach);
     const int lo = max((int)((float)a.eta * (el * rsqrtf(fmaxf(el, 1e-30f))) - 1e-3f), 0);
@@ -550,7 +550,7 @@ __device__ __forceinline__ void radial_setup64(const WalkArgs& a, RadialSpread<0
     const float rch = a.r_coeff * inv_hf;
     for (int i = lo; i <= hi; ++i, fi += 1.f) {
         const double w = gauss ? radial_w<double>(fabs(__ldg(a.r + i) - d), hpar, 1)
-                               : wp_select(fabs(widen(fi * fi * rch) - dh));
+                               : wp_select(fabs(widen_normal(fi * fi * rch) - dh));
         if (positive(w)) {                  // the support is one run of points
             S += w;
             last = i;
@@ -741,10 +741,19 @@ __device__ __forceinline__ int eps_split(const WalkArgs& a, typename Prec<MODE>:
 // FP32 + FP64-sweep form the deposits are FP32, so the coefficient is formed
 // in FP32 and widened; the photon budget (Phi_j, its losses and their
 // clipping) is FP64.
+// The widening takes the power of two of the bin's unit (unit_base), so that no
+// FP32 value leaves the normal range.
+__device__ __forceinline__ int unit_base(float scale) {      // of 1 / scale, scale a power of two
+    return 0x38000000 + (127 - (int)(__float_as_uint(scale) >> 23)) * (1 << 20);
+}
+__device__ __forceinline__ float bin_units(const double* slot) {
+    const uint2 v = *reinterpret_cast<const uint2*>(slot);
+    return (float)v.y * 4294967296.0f + (float)v.x;
+}
 template <int MODE>
-__device__ __forceinline__ double alpha_at(const WalkArgs& a, const double* ba, int i, float inv_scale) {
+__device__ __forceinline__ double alpha_at(const WalkArgs& a, const double* ba, int i, int unit) {
     if (MODE == 0) return ba[i] * __ldg(a.inv_vol + i);
-    return widen(bin_value_f<MODE>(ba + i, inv_scale) * __ldg(a.inv_volf + i));
+    return widen_scaled(bin_units(ba + i) * __ldg(a.inv_volf + i), unit);
 }
 
 // Flux at r = 0 of a ray with a lone source at jtop and no e, by a whole warp
@@ -754,11 +763,11 @@ __device__ __forceinline__ double alpha_at(const WalkArgs& a, const double* ba, 
 template <int MODE>
 __device__ __forceinline__ double lone_ray(const WalkArgs& a, const double* ba, const double* be, const Scales& sc, int jtop) {
     const int lane = threadIdx.x & 31;
-    const float ia = 1.0f / sc.a;
+    const int ia = unit_base(sc.a);
     const double* h = a.HT + (size_t)jtop * a.nr;
     double s0 = 0.0;
     for (int i = lane; i <= jtop; i += 32)
-        s0 = fma(MODE == 0 ? ba[i] : widen(bin_value_f<MODE>(ba + i, ia)), __ldg(h + i), s0);
+        s0 = fma(MODE == 0 ? ba[i] : widen_scaled(bin_units(ba + i), ia), __ldg(h + i), s0);
     s0 = warp_sum(s0);
     const double phi = bin_value<MODE>(be + jtop, (MODE == 0 ? 1.0 : 1.0 / (double)sc.eps) * (1.0 / (4.0 * PI_D))) - s0;
     return positive(phi) && lane == 0 ? phi * __ldg(a.inv_r2 + jtop) : 0.0;
@@ -773,8 +782,7 @@ __device__ __forceinline__ double lone_ray(const WalkArgs& a, const double* ba, 
 // bee[i] the limit A / e (else infinity).
 template <int MODE>
 __device__ __forceinline__ void prepare_ray(const WalkArgs& a, double* ba, double* bee, const Scales& sc, int jtop) {
-    const int lane = threadIdx.x & 31;
-    const float ia = 1.0f / sc.a, ie = 1.0f / sc.e;
+    const int lane = threadIdx.x & 31, ia = unit_base(sc.a), ie = unit_base(sc.e);
     for (int base = 0; base < jtop; base += 32) {
         const int i = base + lane;
         double A = 0.0, Q = 0.0;
@@ -827,8 +835,7 @@ __device__ __forceinline__ double sweep_ray(const WalkArgs& a, const double* ba,
     for (uint64_t w = o0; w; w &= w - 1) { const int j = __ffsll((long long)w) - 1; be[j] = bin_value<MODE>(be + j, f4pi); }
     for (uint64_t w = o1; w; w &= w - 1) { const int j = 64 + __ffsll((long long)w) - 1; be[j] = bin_value<MODE>(be + j, f4pi); }
     double* ph = be;                                              // Eq. 12
-    const int jtop = farthest(m0, m1);
-    const float ia = 1.0f / sc.a;
+    const int jtop = farthest(m0, m1), ia = unit_base(sc.a);
     double a_hi = ready ? 0.0 : alpha_at<MODE>(a, ba, jtop, ia);
     for (int i = jtop - 1; i >= 0; --i) {
         double A = ba[i];
@@ -1586,7 +1593,7 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE, 
         const int b0 = ray * nr + (int)(pk & 0x7fu);
         const real* wc = &nb.w[0][src];
         if constexpr (MODE == 0) {
-            const double c = widen((float)(ec & 0xffffu));
+            const double c = widen_normal((float)(ec & 0xffffu));
             const double ca = c * nb.a[kc], ce = use_e ? c * nb.e[kc] : 0.0;
             const double d = wc[0], hpar = wc[32];
             for (int j = 0; j < npts; ++j) {
