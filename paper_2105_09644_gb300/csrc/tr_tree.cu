@@ -77,6 +77,11 @@ enum { B_M, B_X, B_Y, B_Z, B_ALPHA, B_EPS, B_E, B_MION, B_FIELDS };
 constexpr int BUILD_PAD = BUILD_NT + BUILD_NT / 8;
 __device__ __forceinline__ int padded(int i) { return i + (i >> 3); }
 
+// x > 0, and not NaN, by its bits (1 .. those of infinity).
+__device__ __forceinline__ bool above_zero(double x) {
+    return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
+}
+
 // Centre of mass m p / m of a cell at p (a half integer): p itself unless the
 // rounding of the product moves the quotient to a neighbour, which its exact
 // residual r decides: |r| / m below half an ulp of p.  Two FP64 instructions
@@ -84,7 +89,7 @@ __device__ __forceinline__ int padded(int i) { return i + (i >> 3); }
 __device__ __forceinline__ double cell_centre(double m, float pf, double& mp) {
     const double p = widen_normal(pf);
     mp = __dmul_rn(m, p);
-    if (!(__double2hiint(m) > 0x10000000)) return m > 0.0 ? __ddiv_rn(mp, m) : p;   // tiny or no mass
+    if ((uint32_t)__double2hiint(m) - 0x10000000u >= 0x6ff00000u) return m > 0.0 ? __ddiv_rn(mp, m) : p;   // tiny, no or no finite mass
     const double r = fabs(fma(-m, p, mp));
     const int e = (int)(__float_as_uint(pf) >> 23) - 127;      // 2^e <= p
     const double half_ulp = __hiloint2double(__double2hiint(m) + ((e - 53) << 20), __double2loint(m));   // m 2^(e-53)
@@ -132,11 +137,12 @@ __global__ void __launch_bounds__(BUILD_NT, 3) k_build(BuildArgs a) {
             nd.cmx = cell_centre(nH, (float)ix + 0.5f, sx);
             nd.cmy = cell_centre(nH, (float)iy + 0.5f, sy);
             nd.cmz = cell_centre(nH, (float)iz + 0.5f, sz);
-            const bool rec = __double_as_longlong(net) > 0;
+            // (neither where a cell's rates are not numbers: max(NaN, 0) = 0)
+            const bool rec = above_zero(net), emits = above_zero(-net);
             nd.alpha = rec ? net : 0.0;
-            nd.eps = rec ? 0.0 : fabs(net);
+            nd.eps = emits ? -net : 0.0;
             nd.e = use_e ? ep * a.invEu : 0.0;
-            const bool lit = __double_as_longlong(ep) > 0;
+            const bool lit = above_zero(ep);
             nd.mion = lit ? nH : 0.0;
             a.n64[id] = nd;
             f64[B_M][k] = nH; f64[B_X][k] = sx; f64[B_Y][k] = sy; f64[B_Z][k] = sz;
@@ -147,7 +153,7 @@ __global__ void __launch_bounds__(BUILD_NT, 3) k_build(BuildArgs a) {
                 q.m = nf;
                 q.ox = 0.f; q.oy = 0.f; q.oz = 0.f;
                 q.alpha = rec ? wf : 0.f;
-                q.eps = rec ? 0.f : wf;
+                q.eps = emits ? wf : 0.f;
                 q.e = use_e ? (float)nd.e : 0.f;
                 q.mion = lit ? nf : 0.f;
                 a.n32[id] = q;
@@ -158,7 +164,7 @@ __global__ void __launch_bounds__(BUILD_NT, 3) k_build(BuildArgs a) {
                 if (differs(nd.cmx, widen_normal(px)) || differs(nd.cmy, widen_normal(py)) || differs(nd.cmz, widen_normal(pz))) {
                     const double ex = fabs(widen_normal(px) - nd.cmx), ey = fabs(widen_normal(py) - nd.cmy),
                                  ez = fabs(widen_normal(pz) - nd.cmz);
-                    kap = __double2float_ru(fmax(ex, fmax(ey, ez)));
+                    kap = fmaxf(kap, __double2float_ru(fmax(ex, fmax(ey, ez))));   // (not NaN)
                 }
             }
         } else {
