@@ -111,16 +111,6 @@ __device__ __forceinline__ double warp_sum(double v) {
 // schedulers from one CTA of an SM to the next, and conversions and
 // comparisons go to the integer units.
 
-// 1/a in FP64 for a normal a > 0: the hardware's approximation (measured: off
-// by 2^-19.9 at most) and one step of third order, y (1 + e + e^2) with e = 1 -
-// a y (measured: within 2^-52).  Three FP64 instructions.
-__device__ __forceinline__ double recip(double a) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double e = fma(-a, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
 // The nearest float towards zero of a double in the float range (bounds only).
 __device__ __forceinline__ float narrow(double a) {
     return __uint_as_float(((uint32_t)__double2hiint(a) - 0x38000000u) << 3 | (uint32_t)__double2loint(a) >> 29);
