@@ -32,6 +32,7 @@
 // without radial points, and a separate instantiation for non-default
 // kernels and boundaries.
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "tr_internal.cuh"
@@ -2050,9 +2051,15 @@ WalkArgs make_args(const tr_tree* t) {
     return a;
 }
 
+// A kernel's limit on dynamic shared memory is one value for all threads of the
+// process; it is set for each launch and each query of a fit, so both hold this
+// lock from there on.
+std::mutex g_smem_limit_mu;
+
 template <int NT, typename K>
 tr_status launch_persistent(K kernel, size_t smem, const WalkArgs* jobs, const int64_t* job_end, int n_jobs,
                             int64_t total, unsigned int* counter, cudaStream_t st) {
+    std::lock_guard<std::mutex> lock(g_smem_limit_mu);
     tr_status s = cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                              "cudaFuncSetAttribute(smem)");
     if (s != TR_OK) return s;
@@ -2073,6 +2080,7 @@ tr_status launch_persistent(K kernel, size_t smem, const WalkArgs* jobs, const i
 template <int NT, typename K>
 int resident_ctas(K kernel, size_t smem) {
     int per_sm = 0;
+    std::lock_guard<std::mutex> lock(g_smem_limit_mu);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem) != cudaSuccess) {
         cudaGetLastError();
@@ -2336,6 +2344,7 @@ tr_status sweep_run(const tr_rays* r, double* F, double* e, uint8_t* ion, cudaSt
     const size_t smem = (size_t)(r->use_e ? 3 : 2) * r->npix * r->nr * 8 + sweep_scratch_bytes(r->npix, r->nr);
     auto kern = r->mode == 0 ? k_sweep_stored<0, SWEEP_NT>
                              : (r->mode == 1 ? k_sweep_stored<1, SWEEP_NT> : k_sweep_stored<2, SWEEP_NT>);
+    std::lock_guard<std::mutex> lock(g_smem_limit_mu);
     tr_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                              "cudaFuncSetAttribute(sweep smem)");
     if (s != TR_OK) return s;
