@@ -1355,11 +1355,12 @@ __device__ __forceinline__ double block_sum(double v, double* red, int turn) {
     return t;                                                      // valid in thread 0
 }
 
-// One CTA of NT threads per target (persistent over targets).  Each step
-// pops NT/8 opened nodes and evaluates their NT children, one per thread.
-// Per-thread walk counters go to the job's counters (one atomic per warp).
+// Per-thread walk counters go to the job's counters (one atomic per warp).  A
+// thread counts at most some 3e7 table entries for one target (512^3, every cell
+// and its seven mirror images accepted), so 32 bits hold those of 64.
+constexpr unsigned FLUSH_TARGETS = 64;
 struct WalkCounters {
-    unsigned vis = 0, acc = 0, ent = 0;     // (flushed before they can wrap)
+    unsigned vis = 0, acc = 0, ent = 0;     // (flushed every FLUSH_TARGETS targets, before they can wrap)
     unsigned fb_mac = 0, fb_dep = 0;        // FP32 forms: decisions re-taken in FP64
 };
 
@@ -1703,7 +1704,7 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
         const int j = s_j;
         const int64_t qg = (int64_t)s_q;
         if (j < 0) break;
-        if (cur >= 0 && (j != cur || ++done >= 4096u)) { flush_counters(a, cnt); done = 0; }
+        if (cur >= 0 && (j != cur || ++done >= FLUSH_TARGETS)) { flush_counters(a, cnt); done = 0; }
         if (j != cur) {                                          // load the job (uniform over the CTA)
             __syncthreads();
             const int* src = reinterpret_cast<const int*>(jobs + j);
