@@ -426,47 +426,44 @@ __device__ __forceinline__ T radius_at(int i, T coef, const double* tab) {
     else return (T)(i * i) * coef;
 }
 
-// W_p normalisation of an accepted node: the support of the kernel on the
-// evaluation points and 1/S.  FP32 forms (dtol = bound on the error of d):
-// returns true when a discontinuous choice -- d beyond the last point or
+// W_p normalisation of an accepted node in the FP32 forms: the support of the
+// kernel on the evaluation points and 1/S.  dtol bounds the error of d; returns
+// true when a discontinuous choice -- d beyond the last point or
 // not, or a support that is empty or holds only points within rounding of
 // its edge (the normalisation then jumps between one point and the linear
 // split) -- is not settled in FP32; radial_setup_exact then takes it in FP64.
 template <int MODE, int W>
 __device__ __forceinline__ bool radial_setup(const WalkArgs& a, RadialSpread<MODE>& n, float d, int s, float* wcol, int gauss,
                                              float dtol) {
-    using real = float;
     const int nr = a.nr;
-    const real rc = (MODE == 0) ? (real)a.r_coef : (real)a.r_coeff;
-    n.b = real(1); n.lng = false;
-    const real rlast = radius_at<real>(nr - 1, rc, a.r);
+    const float rc = a.r_coeff;
+    n.b = 1.f; n.lng = false;
+    const float rlast = radius_at<float>(nr - 1, rc, a.r);
     if (d >= rlast) {
-        n.lo = nr - 1; n.npts = 1; wcol[0] = real(1);
-        return MODE != 0 && (float)d - dtol < (float)rlast;
+        n.lo = nr - 1; n.npts = 1; wcol[0] = 1.f;
+        return d - dtol < rlast;
     }
-    if (MODE != 0 && (float)d + dtol >= (float)rlast) return true;
-    const real h = (real)s, inv_h = real(1) / h;
-    const real hpar = gauss ? h : inv_h;
-    const real reach = real(0.8661) * h + (real)dtol;
-    const real dlo = d > reach ? d - reach : real(0);
+    if (d + dtol >= rlast) return true;
+    const float h = (float)s, inv_h = 1.f / h;
+    const float hpar = gauss ? h : inv_h;
+    const float reach = 0.8661f * h + dtol;
+    const float dlo = d > reach ? d - reach : 0.f;
     // floor / ceil of the support's index bounds (i = eta sqrt(2 r), Eq. 4),
-    // from approximate FP32 roots in both forms and a margin above their
-    // error: it only widens the range by a point whose weight is zero, and
-    // the weights themselves are computed in the form's precision
-    const float el = 2.f * (float)dlo, eh = 2.f * (float)(d + reach);
+    // from approximate roots and a margin above their error: it only widens the
+    // range by a point whose weight is zero
+    const float el = 2.f * dlo, eh = 2.f * (d + reach);
     const int lo = max((int)((float)a.eta * (el * rsqrtf(fmaxf(el, 1e-30f))) - 1e-3f), 0);
     const int hi = min((int)((float)a.eta * (eh * rsqrtf(eh)) + 1.001f), nr - 1);
-    real S = real(0);
+    float S = 0.f;
     int cnt = 0, last = lo - 1;
-    real near = real(1e30);                 // the closest point
-    real* col = wcol;
+    float near = 1e30f;                     // the closest point
+    float* col = wcol;
     float fi = (float)lo;
     for (int i = lo; i <= hi; ++i, fi += 1.f) {
-        const real ri = MODE == 0 ? radius_at<real>(i, rc, a.r) : (real)(fi * fi) * rc;
-        const real dist = fabs(ri - d);
-        const real w = radial_w<real>(dist, hpar, gauss);
-        if (MODE != 0) near = fmin(near, dist);
-        if (w > real(0)) {                  // the support is one run of points
+        const float dist = fabs((fi * fi) * rc - d);
+        const float w = radial_w<float>(dist, hpar, gauss);
+        near = fmin(near, dist);
+        if (w > 0.f) {                      // the support is one run of points
             S += w;
             last = i;
             if (cnt < W) *col = w;
@@ -474,23 +471,21 @@ __device__ __forceinline__ bool radial_setup(const WalkArgs& a, RadialSpread<MOD
             ++cnt;
         }
     }
-    if (MODE != 0) {
-        // a point whose kernel argument lies within xtol of sqrt3/2 may fall
-        // on the other side of the support's edge in FP64; that matters when
-        // no point is surely inside, i.e. when the closest one is not
-        const float xtol = 2.f * (dtol + U32 * (2.f * (float)d + (float)reach)) * (float)inv_h + 4.f * U32;
-        const float x = (float)(near * inv_h) - (float)S3H_D;
-        if (!(x < -xtol) && x <= xtol) return true;
-    }
+    // a point whose kernel argument lies within xtol of sqrt3/2 may fall on the
+    // other side of the support's edge in FP64; that matters when no point is
+    // surely inside, i.e. when the closest one is not
+    const float xtol = 2.f * (dtol + U32 * (2.f * d + reach)) * inv_h + 4.f * U32;
+    const float x = near * inv_h - (float)S3H_D;
+    if (!(x < -xtol) && x <= xtol) return true;
     if (cnt > 0) {
-        n.lo = last - cnt + 1; n.npts = cnt; n.b = real(1) / S;
+        n.lo = last - cnt + 1; n.npts = cnt; n.b = 1.f / S;
         if (cnt > W) { n.lng = true; wcol[0] = d; wcol[32] = hpar; }
         return false;
     }
-    int i = min(max((int)floorf((float)a.eta * sqrtf(2.f * (float)d)), 0), nr - 2);   // a guess, corrected below
-    while (i + 1 < nr - 1 && radius_at<real>(i + 1, rc, a.r) <= d) ++i;
-    while (i > 0 && radius_at<real>(i, rc, a.r) > d) --i;
-    const real ra = radius_at<real>(i, rc, a.r), rb = radius_at<real>(i + 1, rc, a.r);
+    int i = min(max((int)floorf((float)a.eta * sqrtf(2.f * d)), 0), nr - 2);   // a guess, corrected below
+    while (i + 1 < nr - 1 && radius_at<float>(i + 1, rc, a.r) <= d) ++i;
+    while (i > 0 && radius_at<float>(i, rc, a.r) > d) --i;
+    const float ra = radius_at<float>(i, rc, a.r), rb = radius_at<float>(i + 1, rc, a.r);
     n.lo = i; n.npts = 2;
     wcol[0] = (rb - d) / (rb - ra);
     wcol[32] = (d - ra) / (rb - ra);
@@ -513,7 +508,7 @@ __device__ __forceinline__ int bracket_d(const double* r, int nr, int eta, doubl
     return i;
 }
 
-// The same in FP64, settled always.  Bound by the FP64 units, so six FP64
+// The W_p normalisation in FP64, settled always.  Bound by the FP64 units, so six FP64
 // instructions per point (the kernel's argument is one add, r_i / h being exact
 // in FP32; four for the kernel, one for the sum) and none for the index bounds,
 // comparisons and conversions: plain FP64 turbulent64 92 -> 70 ms, Stroemgren
@@ -563,9 +558,9 @@ __device__ __forceinline__ void radial_setup64(const WalkArgs& a, RadialSpread<0
 }
 
 // FP32 forms: the radial set-up of an accepted node taken on its FP64
-// distance d, when radial_setup could not settle it.  Only the supports
-// that FP32 left open reach here (at most two points, both at the edge, or
-// consecutive points, or the linear split between the points bracketing d.
+// distance d, when radial_setup could not settle it: a d within rounding of the
+// last point, or a support that FP32 left open (at most two points, both at its
+// edge, or none).  Few weights are stored explicitly: one point, two
 // consecutive points, or the linear split between the points bracketing d.
 template <int MODE>
 __device__ void radial_setup_exact(const WalkArgs& a, RadialSpread<MODE>& n, double d, int s,
@@ -592,7 +587,7 @@ __device__ void radial_setup_exact(const WalkArgs& a, RadialSpread<MODE>& n, dou
     }
     if (cnt == 1) { n.lo = first; n.npts = 1; wcol[0] = 1.f; return; }
     if (cnt == 2) { n.lo = first; n.npts = 2; wcol[0] = (float)(w0 / S); wcol[32] = (float)(w1 / S); return; }
-    if (cnt > 2) {                          // not reached (FP32 saw no point well inside); FP32 weights
+    if (cnt > 2) {                          // (only beside the last point) FP32 weights, evaluated per ray
         n.lo = first; n.npts = cnt; n.lng = true; n.b = (float)(1.0 / S);
         wcol[0] = (float)d; wcol[32] = (float)hpar;
         return;
@@ -1647,6 +1642,12 @@ constexpr int STACK_CAP = 512;
 constexpr int FIFO_MAX = 64;
 constexpr int STACK_RESERVE = 7 * (MAX_LEVELS - 1);
 
+// The limit on a target's ray bins and node buffer: what these leave of a CTA's
+// shared memory.  Fixed figures, so that the calls that are refused do not
+// change with the kernels; the smallest CTA fits beside the largest bins
+// (asserted in walk_body), the larger ones where there is room.
+constexpr size_t OWN_SMEM_F32 = 19072, OWN_SMEM_F64 = 40512;
+
 // A CTA of NT threads per target.  Walk step: take NT/8 opened nodes from the
 // shared buffer, evaluate their NT children, one per thread; opened children
 // go back into the buffer, accepted ones with something to map to a list.  When
@@ -1677,9 +1678,10 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
     __shared__ __align__(16) WalkArgs s_a;                       // the current job
     __shared__ NodeBatch<MODE, MAXW<MODE, SLIM>> s_nb[NW];
     __shared__ uint32_t s_acc[acc_cap<NT, SLIM>()];
+    constexpr size_t own = sizeof s_nb + sizeof s_acc + sizeof s_a + sizeof s_red + 32;
+    static_assert(NT != 128 || own <= (MODE == 0 ? OWN_SMEM_F64 : OWN_SMEM_F32), "the largest bins leave room for this CTA");
     // (228 KB an SM, 1 KB of it the system's per CTA; 48 rays of 59 points, alpha and eps)
-    static_assert(MODE == 0 || NT != 128 ||
-                      sizeof s_nb + sizeof s_acc + sizeof s_a + sizeof s_red + 32 <= 228 * 1024 / 4 - 1024 - 48 * 59 * 16 - STACK_CAP * 4,
+    static_assert(MODE == 0 || NT != 128 || own <= 228 * 1024 / 4 - 1024 - 48 * 59 * 16 - STACK_CAP * 4,
                   "four targets of a 256^3 grid fit an SM");
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const WalkArgs& a = s_a;
@@ -2150,15 +2152,16 @@ template <int MODE, int OUT, bool VAR>
 tr_status launch_sized(BinShape b, const WalkArgs* jobs, const int64_t* job_end, int n_jobs, int64_t total,
                        unsigned int* counter, cudaStream_t st) {
     auto* const k5 = k_walk<MODE, OUT, 128, 5, VAR>;
-    if constexpr (OUT == OUT_CD) return launch_persistent<128>(k5, b.smem, jobs, job_end, n_jobs, total, counter, st);
-    const CtaKind kind = pick_cta<MODE, OUT, VAR>(b.smem, b.npix).kind;
-    if constexpr (OUT == OUT_FUSED && MODE != 0)
-        if (kind == K6) return launch_persistent<128>(k_walk<MODE, OUT, 128, 6, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
-    if constexpr (OUT == OUT_FUSED && MODE != 0)
-        if (kind == K512_SLIM) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR, true>, b.smem, jobs, job_end, n_jobs, total, counter, st);
-    if constexpr (MODE != 0)
-        if (kind == K512) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
-    if (kind == K256) return launch_persistent<256>(k_walk<MODE, OUT, 256, 2, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
+    if constexpr (OUT != OUT_CD) {                            // (column densities: few bins, 128 threads always)
+        const CtaKind kind = pick_cta<MODE, OUT, VAR>(b.smem, b.npix).kind;
+        if constexpr (OUT == OUT_FUSED && MODE != 0)
+            if (kind == K6) return launch_persistent<128>(k_walk<MODE, OUT, 128, 6, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
+        if constexpr (OUT == OUT_FUSED && MODE != 0)
+            if (kind == K512_SLIM) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR, true>, b.smem, jobs, job_end, n_jobs, total, counter, st);
+        if constexpr (MODE != 0)
+            if (kind == K512) return launch_persistent<512>(k_walk<MODE, OUT, 512, 1, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
+        if (kind == K256) return launch_persistent<256>(k_walk<MODE, OUT, 256, 2, VAR>, b.smem, jobs, job_end, n_jobs, total, counter, st);
+    }
     return launch_persistent<128>(k5, b.smem, jobs, job_end, n_jobs, total, counter, st);
 }
 
@@ -2180,11 +2183,6 @@ tr_status launch_jobs_v(int mode, int out, BinShape b, const WalkArgs* jobs, con
         return launch_mode<1, VAR>(out, b, jobs, job_end, n_jobs, total, counter, st);
     return launch_mode<2, VAR>(out, b, jobs, job_end, n_jobs, total, counter, st);
 }
-
-// Shared memory of a CTA that is not for ray bins and the node buffer: what
-// the 512-thread FP32 and 256-thread FP64 walks take at most, and so the
-// limit on a target's bins whichever CTA size is picked.
-constexpr size_t OWN_SMEM_F32 = 19072, OWN_SMEM_F64 = 40512;
 
 // The one refusal of a walk: bins that no CTA can hold.
 tr_status check_bins(int mode, int out, size_t smem) {
