@@ -2210,9 +2210,10 @@ tr_status launch_jobs(int mode, int out, bool var, BinShape b, const WalkArgs* j
 }
 
 // Targets that an SM holds at once in the fused walk of a form.
+template <bool VAR>
 int targets_per_sm(int mode, BinShape b) {
-    return (mode == 0 ? pick_cta<0, OUT_FUSED, false>(b.smem, b.npix)
-            : mode == 1 ? pick_cta<1, OUT_FUSED, false>(b.smem, b.npix) : pick_cta<2, OUT_FUSED, false>(b.smem, b.npix)).per_sm;
+    return (mode == 0 ? pick_cta<0, OUT_FUSED, VAR>(b.smem, b.npix)
+            : mode == 1 ? pick_cta<1, OUT_FUSED, VAR>(b.smem, b.npix) : pick_cta<2, OUT_FUSED, VAR>(b.smem, b.npix)).per_sm;
 }
 constexpr int BATCH_WAVES = 4;              // targets per resident target below which a batch's group is too small
 
@@ -2282,7 +2283,8 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
     for (int i = 0; i < n; ++i)
         if (count[i] > 0) {
             const size_t m = walk_smem(trees[i]);
-            items.push_back({i, targets_per_sm(mode, {m, trees[i]->npix}), m});
+            const BinShape b{m, trees[i]->npix};
+            items.push_back({i, uses_variants(trees[i]) ? targets_per_sm<true>(mode, b) : targets_per_sm<false>(mode, b), m});
         }
     std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.per_sm > y.per_sm; });
     int dev = 0, sms = 0;
