@@ -117,7 +117,9 @@ typedef struct {
  * ndot: extra per-cell EUV emission (photons s^-1), may be NULL.
  * e_prev: per-cell EUV energy density (erg cm^-3) from a previous pass, may
  *         be NULL; it enters the IF MAC (ionised mass, Sec. 2.4) and zeta_d
- *         (Eq. 17), and seeds the iteration of tr_solve (Sec. 2.6). */
+ *         (Eq. 17), and seeds the iteration of tr_solve (Sec. 2.6).  Values
+ *         >= 0 are meant; -0 is 0, and where a node's sum is below 0 the FP64
+ *         form maps it with its sign and the FP32 forms as 0. */
 typedef struct {
     int32_t N;
     double box_lo[3];       /* low corner of the box, cm */

@@ -23,14 +23,14 @@
 // for the emission eps), with shared-memory atomics into the ray bins: FP64
 // adds in the FP64 form, exact 64-bit fixed point in the FP32 forms.
 // Sweep (Sec. 2.5, Eq. 12-17): each ray is swept far to near (FP64 and
-// FP32 + FP64-sweep forms: FP64 arithmetic, a lane per ray of few sources
-// and a lane pair per other ray; FP32 + double-FP32-sweep form: FP32 losses,
-// double-FP32 budgets, a lane per source or a pair per ray) and the CTA sums
-// the rays (Eq. 18).
-// Variants: CTAs of 128, 256 or 512 threads by the room that the bins leave,
-// a dump mode keeping the raw bins and accepted ids, a column-density mode
-// without radial points, and a separate instantiation for non-default
-// kernels and boundaries.
+// FP32 + FP64-sweep forms: FP64 arithmetic, a lane per emitting point while a
+// target has few, else a lane pair per ray, a warp per ray with a lone source;
+// FP32 + double-FP32-sweep form: FP32 losses, double-FP32 budgets, a lane per
+// source or a pair per ray) and the CTA sums the rays (Eq. 18).
+// Variants: CTAs of 128, 256 or 512 threads by the room that the bins leave
+// (pick_cta), a dump mode keeping the raw bins and accepted ids, a
+// column-density mode without radial points, and a separate instantiation for
+// non-default kernels and boundaries.
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -2215,7 +2215,10 @@ int targets_per_sm(int mode, BinShape b) {
     return (mode == 0 ? pick_cta<0, OUT_FUSED, VAR>(b.smem, b.npix)
             : mode == 1 ? pick_cta<1, OUT_FUSED, VAR>(b.smem, b.npix) : pick_cta<2, OUT_FUSED, VAR>(b.smem, b.npix)).per_sm;
 }
-constexpr int BATCH_WAVES = 4;              // targets per resident target below which a batch's group is too small
+// Targets per resident target below which a batch's group is too small to launch
+// alone.  0 to 16 measured the same on seven batches of two to nine trees (16^3 to
+// 128^3, N_PIX 48 and 192, a slice of 256^3), one launch for all 3 to 90% slower.
+constexpr int BATCH_WAVES = 4;
 
 bool uses_variants(const tr_tree* t) {
     return t->p.kernel_alpha != TR_KERNEL_WP || t->p.kernel_eps != TR_EPS_WF3 || t->p.bc != TR_BC_ISOLATED;
@@ -2265,7 +2268,7 @@ tr_status walk_batch_run(const tr_tree* const* trees, const int64_t* first, cons
     // Jobs by the number of targets that an SM holds at once with each tree's
     // own ray bins, one launch for each: a tree with N_PIX 192 would otherwise
     // set the shared memory, and so the warps per SM, of every target (two 64^3
-    // and two 32^3 trees, one with N_PIX 192: 141 -> 75 ms).  A group too small
+    // and two 32^3 trees, one with N_PIX 192: 141 -> 76 ms).  A group too small
     // to fill the GPU a few times over joins the next with larger bins.
     struct Item { int tree, per_sm; size_t smem; };
     const int mode = trees[0]->mode;
