@@ -275,10 +275,10 @@ __device__ __forceinline__ bool bin_nonzero(const double* slot) {
 
 // FP32 forms: add v >= +0 (in units of the bin, below 2^62; the caller sees to
 // it: the sign bit would be read as part of the exponent, so that -0 would add
-// 2^33 units), rounded down to an integer, to a bin.  Integer placement of the significand rather than two
-// float-to-integer conversions: those share a pipe of 16 lanes per SM and
-// clock (turbulent128, double-FP32 form: 232 -> 226 ms; the unconditional
-// second atomic 226 -> 217 ms).
+// 2^33 units), rounded down to an integer, to a bin.  Integer placement of the
+// significand rather than two float-to-integer conversions: those share a pipe
+// of 16 lanes per SM and clock (turbulent128, double-FP32 form: 232 -> 226 ms;
+// the unconditional second atomic 226 -> 217 ms).
 __device__ __forceinline__ void bin_add_units(double* slot, float v) {
     unsigned* w = reinterpret_cast<unsigned*>(slot);
     // the 24-bit significand placed in 64 bits by one widening multiply
@@ -1257,17 +1257,17 @@ __device__ __forceinline__ double sweep_groups(const WalkArgs& a, const double* 
 // rotates which warps take the work from target to target.
 // FP64 sweeps (FP64 form and FP32 + FP64-sweep form): rays with a lone source
 // by a warp each (lone_ray).  Of the others, while their points fill at most
-// group_lanes_max lanes, all warps ready the rays
-// (prepare_ray) and sweep them a lane per point (sweep_group64; more than
-// GROUP_MAX points: lane pairs): the fewest FP64 instructions in a row, and the
-// target's time is that chain.  Beyond that the FP64 units are what is short,
+// group_lanes_max lanes, all warps ready the rays (prepare_ray) and sweep them a
+// lane per point (sweep_group64; more than GROUP_MAX points: lane pairs): the
+// fewest FP64 instructions in a row, and the target's time is that chain.  Beyond that the FP64 units are what is short,
 // and lane pairs, 16 rays of like load to a warp, take fewest in all (a lane
 // for a point that the sweep has not reached costs as much as a busy one).
 // The line lies at 128 lanes for up to 96 rays (turbulent128 278 -> 236 ms
 // with it, 275 with pairs only, 251 with 64 lanes) and at 4/3 of a lane per ray
-// beyond (N_PIX 192, 64^3, 10 sources: 23.1 ms with 256 lanes, 23.9 with 128; AMR 64^3
-// 24 ms, 35 with groups only).  Coefficients computed within the chain where lane pairs
-// sweep: 505 -> 492 ms for 10^4 sources at 128^3 (its FP64 units are busy).
+// beyond (N_PIX 192, 64^3, 10 sources: 23.1 ms with 256 lanes, 23.9 with 128;
+// AMR 64^3 24 ms, 35 with groups only).  Coefficients computed within the chain
+// where lane pairs sweep: 505 -> 492 ms for 10^4 sources at 128^3 (its FP64
+// units are busy).
 // Double-FP32 sweep: lane groups up to GROUP_MEAN_MAX points per lit ray on
 // average (sweep_groups), lane pairs beyond (sweep_ray_group).  The choices
 // depend only on the bins and N_PIX, so a target's rays are swept alike in a CTA
