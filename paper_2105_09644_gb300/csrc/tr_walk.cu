@@ -384,15 +384,18 @@ __device__ __forceinline__ double exact_d2(const WalkArgs& a, int64_t nid, float
 // the lane keeps in its column of the warp's NodeBatch, times b; a support
 // of more than MAXW points is evaluated again for each ray instead (`lng`:
 // column entries 0 and 1 then hold d and the kernel's size argument).
-// Kernel values kept per node.  FP32: 7, so that a 128-thread CTA takes 9.7 KB
-// beside its ray bins and as many targets fit an SM as should: five at 33 KB of
-// bins (N_PIX 48, N_R 43; with 12 values only four: 225 -> 253 ms), four at 45
-// KB (N_R 59; with 8 only three, by 256 bytes: a 256^3 grid with 100 sources
-// 406 -> 329 ms per 10^6 targets, headline form).  A longer support, met by the
-// few nodes with edges of 32 cells and more, costs its evaluation again per
-// ray.  FP64: 12, evaluating again costs more.
-// SLIM: the 512-thread CTA beside bins of 190 to 199 KB (see pick_cta).
-template <int MODE, bool SLIM = false> constexpr int MAXW = MODE == 0 ? 12 : (SLIM ? 6 : 7);
+// Kernel values kept per node.  A longer support, met by the few nodes with
+// edges of 32 cells and more, costs its evaluation again per ray.
+// FP64: 12, evaluating again costs more.  FP32: 7, so that a 128-thread CTA
+// takes 9.7 KB beside its ray bins and as many targets fit an SM as should: five
+// at 33 KB of bins (N_PIX 48, N_R 43; with 12 values only four: 225 -> 253 ms),
+// four at 45 KB (N_R 59; with 8 only three, by 256 bytes: a 256^3 grid with 100
+// sources 406 -> 329 ms per 2^20 targets, headline form).  8 where six CTAs fit
+// (the bins leave room), and for the other radial kernels, whose evaluation is
+// an exponential and a division (W_g headline walk of 32^3: 1.82 -> 1.72 ms).  6
+// in the slim 512-thread CTA (see pick_cta).
+template <int MODE, int NT, int CTAS, bool VAR, bool SLIM>
+constexpr int MAXW = MODE == 0 ? 12 : (SLIM ? 6 : (NT == 128 && (CTAS == 6 || VAR) ? 8 : 7));
 
 template <int MODE>
 struct RadialSpread {
@@ -513,6 +516,7 @@ __device__ __forceinline__ int bracket_d(const double* r, int nr, int eta, doubl
 // in FP32; four for the kernel, one for the sum) and none for the index bounds,
 // comparisons and conversions: plain FP64 turbulent64 92 -> 70 ms, Stroemgren
 // 32^3 7.5 -> 5.6 ms.
+template <int W>
 __device__ __forceinline__ void radial_setup64(const WalkArgs& a, RadialSpread<0>& n, double d, int s, double* wcol,
                                                int gauss) {
     const int nr = a.nr;
@@ -540,14 +544,14 @@ __device__ __forceinline__ void radial_setup64(const WalkArgs& a, RadialSpread<0
         if (positive(w)) {                  // the support is one run of points
             S += w;
             last = i;
-            if (cnt < MAXW<0>) *col = w;
+            if (cnt < W) *col = w;
             col += 32;
             ++cnt;
         }
     }
     if (cnt > 0) {
         n.lo = last - cnt + 1; n.npts = cnt; n.b = recip(S);
-        if (cnt > MAXW<0>) { n.lng = true; wcol[0] = d; wcol[32] = hpar; }
+        if (cnt > W) { n.lng = true; wcol[0] = d; wcol[32] = hpar; }
         return;
     }
     const int i = bracket_d(a.r, nr, a.eta, d);
@@ -1511,7 +1515,7 @@ __device__ __forceinline__ void spread_nodes(const WalkArgs& a, NodeBatch<MODE, 
                 if (qv[0] != real(0) || (a.use_e && qv[2] != real(0))) {
                     const int gauss = VAR ? a.kern_a : 0;
                     real* const wcol = &nb.w[0][lane];
-                    if constexpr (MODE == 0) radial_setup64(a, n, d, s, wcol, gauss);
+                    if constexpr (MODE == 0) radial_setup64<W>(a, n, d, s, wcol, gauss);
                     else if (radial_setup<MODE, W>(a, n, d, s, wcol, gauss, dtol))
                         radial_setup_exact<MODE>(a, n, exact_d(), s, wcol, gauss);
                     alpha = qv[0];
@@ -1659,7 +1663,7 @@ constexpr size_t OWN_SMEM_F32 = 19072, OWN_SMEM_F64 = 40512;
 // before, left a third of the lanes idle and took turbulent128 from 217 to
 // 328 ms in the double-FP32 form (99 k to 62 k warp instructions per target
 // in the headline form).
-template <int MODE, int OUT, int NT, bool VAR, bool SLIM>
+template <int MODE, int OUT, int NT, bool VAR, int W, bool SLIM>
 __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, const int64_t* __restrict__ job_end,
                                           int n_jobs, unsigned int* counter) {
     using real = typename Prec<MODE>::real;
@@ -1676,12 +1680,12 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
     __shared__ int s_j;
     __shared__ int s_nacc;
     __shared__ __align__(16) WalkArgs s_a;                       // the current job
-    __shared__ NodeBatch<MODE, MAXW<MODE, SLIM>> s_nb[NW];
+    __shared__ NodeBatch<MODE, W> s_nb[NW];
     __shared__ uint32_t s_acc[acc_cap<NT, SLIM>()];
     constexpr size_t own = sizeof s_nb + sizeof s_acc + sizeof s_a + sizeof s_red + 32;
     static_assert(NT != 128 || own <= (MODE == 0 ? OWN_SMEM_F64 : OWN_SMEM_F32), "the largest bins leave room for this CTA");
     // (228 KB an SM, 1 KB of it the system's per CTA; 48 rays of 59 points, alpha and eps)
-    static_assert(MODE == 0 || NT != 128 || own <= 228 * 1024 / 4 - 1024 - 48 * 59 * 16 - STACK_CAP * 4,
+    static_assert(MODE == 0 || NT != 128 || W > 7 || own <= 228 * 1024 / 4 - 1024 - 48 * 59 * 16 - STACK_CAP * 4,
                   "four targets of a 256^3 grid fit an SM");
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const WalkArgs& a = s_a;
@@ -1956,7 +1960,7 @@ __device__ __forceinline__ void walk_body(const WalkArgs* __restrict__ jobs, con
 template <int MODE, int OUT, int NT, int CTAS, bool VAR, bool SLIM = false>
 __global__ void __launch_bounds__(NT, CTAS) k_walk(const WalkArgs* __restrict__ jobs, const int64_t* __restrict__ job_end,
                                                   int n_jobs, unsigned int* counter) {
-    walk_body<MODE, OUT, NT, VAR, SLIM>(jobs, job_end, n_jobs, counter);
+    walk_body<MODE, OUT, NT, VAR, MAXW<MODE, NT, CTAS, VAR, SLIM>, SLIM>(jobs, job_end, n_jobs, counter);
 }
 
 // Unfused sweep over bins stored by the dump walk: one CTA per target.
